@@ -198,7 +198,9 @@ constexpr size_t kPotrfSmem = (size_t)(NB * (NB + 1) + 4 * NB) * 8;   // final c
 // steps: fewer threads per row (8: 5 % slower, 4: 30 % slower on GB300) leave
 // that latency exposed, though each thread then repeats less per-row work.
 // Each step publishes column j of S and row j of Y to shared memory (double
-// buffered, so one barrier per column suffices).  At the end
+// buffered, so one barrier per column suffices), and the pivot's owner its reciprocal: a division
+// in every thread (32 warps, about ten FP64 instructions of 17 clocks each on the SM's one FP64
+// pipe) took longer than that thread's latency (85 -> 75 us per block).  At the end
 // L'[i][j] = S[i][j] / sqrt(d_j) and L'^{-1}[i][c] = Y[i][c] / sqrt(d_i);
 // undoing D gives L = D^-1 L' and Linv = L'^{-1} D, written in FP64.
 template <class AR, int TPR>
@@ -214,6 +216,7 @@ __global__ void __launch_bounds__(NB * TPR) potrf_inv_kernel(double* A, int64_t 
   T* colbuf = reinterpret_cast<T*>(smraw) + NB * (NB + 1);     // [2][NB]: column j of S
   T* rowbuf = colbuf + 2 * NB;                                 // [2][NB]: row j of Y; reused for 1/sqrt(d)
   __shared__ int sc[NB];
+  __shared__ T rcps[2];   // 1 / d_j, double buffered like colbuf
   if (*flag) return;
   const int t = threadIdx.x, i = t / TPR, g = t % TPR;
   if (t < NB) {
@@ -258,6 +261,7 @@ __global__ void __launch_bounds__(NB * TPR) potrf_inv_kernel(double* A, int64_t 
         // from here on the register accumulates Y[i][j] (0 below the diagonal of I)
         cb[i] = v;
         Lf[i][j] = v;
+        if (i == j) rcps[j & 1] = AR::rcp(v);
       }
       if (i == j) {
 #pragma unroll
@@ -272,7 +276,7 @@ __global__ void __launch_bounds__(NB * TPR) potrf_inv_kernel(double* A, int64_t 
       break;
     }
     if (i > j && i < kb) {
-      const T a = AR::mul(cb[i], AR::rcp(d));
+      const T a = AR::mul(cb[i], rcps[j & 1]);
       const int mmax = (i - g) >= 0 ? (i - g) / TPR : -1;   // columns c = g + TPR m <= i
 #pragma unroll
       for (int m = 0; m < EPT; m++) {
@@ -645,34 +649,35 @@ __global__ void __launch_bounds__(256) diag_to_fp64_kernel(double* A, int64_t ld
 }
 
 // Panel solve L21 = A21 Linv_k^T in FP64 on the CUDA cores (the FP64 path), in
-// place, for the rows [k1, n) of the panel columns [k0, k0 + kb).  32 rows per
-// CTA, 128 threads, 4 x 4 outputs per thread (rows ty + 8a, columns tx + 16b);
+// place, for the rows [k1, n) of the panel columns [k0, k0 + kb).  ROWS rows per
+// CTA, 128 threads, ROWS / 8 x 4 outputs per thread (rows ty + 8a, columns tx + 16b);
 // Linv_k is lower triangular, so the K loop runs in four 16-wide segments and
 // segment s only feeds the columns b >= s.
-constexpr int kPanelRows = 32;
-constexpr size_t kPanelSmem = (size_t)(kPanelRows + NB) * (NB + 1) * 8;
+constexpr size_t panel_smem(int rows) { return (size_t)(rows + NB) * (NB + 1) * 8; }
 
+template <int ROWS>
 __global__ void __launch_bounds__(128) panel_solve_kernel(double* A, int64_t lda, int64_t k0, int kb, int64_t k1,
                                                           int64_t n, const double* __restrict__ Lk, const int* flag) {
   extern __shared__ __align__(16) unsigned char smraw[];
   double (*As)[NB + 1] = reinterpret_cast<double (*)[NB + 1]>(smraw);
-  double (*Lt)[NB + 1] = As + kPanelRows;   // Lt[q][j] = Linv_k[j][q]
+  constexpr int AR = ROWS / 8;
+  double (*Lt)[NB + 1] = As + ROWS;   // Lt[q][j] = Linv_k[j][q]
   if (*flag) return;
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int64_t rb = k1 + (int64_t)blockIdx.x * kPanelRows;   // first row of this CTA
+  const int64_t rb = k1 + (int64_t)blockIdx.x * ROWS;   // first row of this CTA
   for (int idx = t; idx < NB * NB; idx += blockDim.x) {
     const int j = idx / NB, q = idx % NB;
     Lt[q][j] = (j < kb && q < kb) ? Lk[j * NB + q] : 0.0;
   }
-  for (int idx = t; idx < kPanelRows * NB; idx += blockDim.x) {
+  for (int idx = t; idx < ROWS * NB; idx += blockDim.x) {
     const int rr = idx / NB, q = idx % NB;
     const int64_t r = rb + rr;
     As[rr][q] = (r < n && q < kb) ? A[r * lda + k0 + q] : 0.0;
   }
   __syncthreads();
-  double acc[4][4];
+  double acc[AR][4];
 #pragma unroll
-  for (int a = 0; a < 4; a++)
+  for (int a = 0; a < AR; a++)
 #pragma unroll
     for (int b = 0; b < 4; b++) acc[a][b] = 0.0;
 #pragma unroll
@@ -680,19 +685,19 @@ __global__ void __launch_bounds__(128) panel_solve_kernel(double* A, int64_t lda
 #pragma unroll 4
     for (int tt = 0; tt < 16; tt++) {
       const int q = 16 * seg + tt;
-      double av[4], lv[4];
+      double av[AR], lv[4];
 #pragma unroll
-      for (int a = 0; a < 4; a++) av[a] = As[ty + 8 * a][q];
+      for (int a = 0; a < AR; a++) av[a] = As[ty + 8 * a][q];
 #pragma unroll
       for (int b = seg; b < 4; b++) lv[b] = Lt[q][tx + 16 * b];
 #pragma unroll
-      for (int a = 0; a < 4; a++)
+      for (int a = 0; a < AR; a++)
 #pragma unroll
         for (int b = seg; b < 4; b++) acc[a][b] = fma(av[a], lv[b], acc[a][b]);
     }
   }
 #pragma unroll
-  for (int a = 0; a < 4; a++) {
+  for (int a = 0; a < AR; a++) {
     const int64_t r = rb + ty + 8 * a;
     if (r >= n) continue;
 #pragma unroll
@@ -986,16 +991,26 @@ cudaError_t launch_potrf_blk(const double* A, int64_t lda, int64_t k0, int kb, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_panel(double* A, int64_t lda, int64_t k0, int kb, int64_t k1, int64_t n, const double* Lk,
-                         const int* flag, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(panel_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kPanelSmem);
+template <int ROWS>
+cudaError_t launch_panel_rows(double* A, int64_t lda, int64_t k0, int kb, int64_t k1, int64_t n, const double* Lk,
+                              const int* flag, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(panel_solve_kernel<ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)panel_smem(ROWS));
   if (e != cudaSuccess) return e;
-  const int64_t blocks = (n - k1 + kPanelDFRowsCTA - 1) / kPanelDFRowsCTA;
+  const int64_t blocks = (n - k1 + ROWS - 1) / ROWS;
   if (blocks <= 0) return cudaSuccess;
-  panel_solve_kernel<<<(unsigned)blocks, 128, kPanelSmem, st>>>(A, lda, k0, kb, k1, n, Lk, flag);
+  panel_solve_kernel<ROWS><<<(unsigned)blocks, 128, panel_smem(ROWS), st>>>(A, lda, k0, kb, k1, n, Lk, flag);
   count_launch();
   return cudaGetLastError();
+}
+
+// 8 rows per CTA while 32-row CTAs would not fill the 152 SMs (each row is 2080 FP64 FMAs on its
+// SM's one FP64 pipe; at n = 1154 the panel takes 15 us instead of 27), 32 rows above, where the
+// 32 KB of Linv_k that every CTA reads would cost more than the balance gains.
+cudaError_t launch_panel(double* A, int64_t lda, int64_t k0, int kb, int64_t k1, int64_t n, const double* Lk,
+                         const int* flag, cudaStream_t st) {
+  return (n - k1) / 32 < 152 ? launch_panel_rows<8>(A, lda, k0, kb, k1, n, Lk, flag, st)
+                             : launch_panel_rows<32>(A, lda, k0, kb, k1, n, Lk, flag, st);
 }
 
 template <int S>
@@ -1038,24 +1053,51 @@ cudaError_t launch_panel_split(int S, double* A, int64_t lda, int64_t k0, int kb
 
 }  // namespace
 
-cudaError_t cholesky_factor(double* A, int64_t n, int64_t lda, double* Linv, int* flag, cudaStream_t st) {
-  cudaError_t err = cudaSuccess;
+// FP64 factorisation.  Look-ahead: panel k's update of the next 64 columns runs on the critical
+// stream, so that the next diagonal factor (one CTA, a dependent chain) starts at once; the rest
+// of the trailing update runs on the low-priority stream beside that factor and its panel.  The
+// rest of panel k - 1 also writes the next columns, so the critical stream waits for it there.
+// Damped solve at n = 1154 / 1274: 2.65 / 3.01 -> 2.52 / 2.69 ms (4.50 / 4.96 before the balanced
+// tiles of the trailing update, the shared pivot reciprocal and the 8-row panels).
+cudaError_t cholesky_factor(gn_handle* h, double* A, int64_t n, int64_t lda, double* Linv, int* flag) {
+  cudaError_t err = ensure_chol_streams(h);
+  if (err != cudaSuccess) return err;
+  cudaStream_t st = h->st, sh = h->st_hi, sl = h->st_lo;
+  auto follow = [](cudaStream_t after, cudaEvent_t e, cudaStream_t before) {
+    const cudaError_t r = cudaEventRecord(e, before);
+    return r != cudaSuccess ? r : cudaStreamWaitEvent(after, e, 0);
+  };
+  if ((err = follow(sh, h->ev_panel, st)) != cudaSuccess) return err;
+  bool rest = false;   // a trailing update is in flight on sl
   for (int64_t k0 = 0; k0 < n; k0 += NB) {
     const int kb = (int)((n - k0) < NB ? (n - k0) : NB);
     if ((err = launch_potrf<Arith64>(A, lda, k0, kb, nullptr, 0, Linv, nullptr, nullptr, nullptr, nullptr, nullptr,
-                                     flag, st)) != cudaSuccess)
+                                     flag, sh)) != cudaSuccess)
       return err;
     const int64_t k1 = k0 + kb;
     if (k1 >= n) break;
     const double* Lk = Linv + (k0 / NB) * NB * NB;
     // panel: A21 <- A21 Linv_k^T
-    if ((err = launch_panel(A, lda, k0, kb, k1, n, Lk, flag, st)) != cudaSuccess) return err;
-    // trailing: A22 -= L21 L21^T (lower)
-    err = dgemm(n - k1, n - k1, kb, -1.0, A + k1 * lda + k0, lda, true, A + k1 * lda + k0, lda, true, 1.0,
-                A + k1 * lda + k1, lda, true, nullptr, st);
-    if (err != cudaSuccess) return err;
+    if ((err = launch_panel(A, lda, k0, kb, k1, n, Lk, flag, sh)) != cudaSuccess) return err;
+    // trailing: A22 -= L21 L21^T (lower), the next panel's columns first
+    const int64_t k2 = k1 + NB < n ? k1 + NB : n;
+    const double* L1 = A + k1 * lda + k0;
+    if (rest && (err = cudaStreamWaitEvent(sh, h->ev_rest, 0)) != cudaSuccess) return err;
+    if (k2 < n && (err = follow(sl, h->ev_panel, sh)) != cudaSuccess) return err;
+    if ((err = dgemm(n - k1, k2 - k1, kb, -1.0, L1, lda, true, L1, lda, true, 1.0, A + k1 * lda + k1, lda, false,
+                     nullptr, sh)) != cudaSuccess)
+      return err;
+    if (k2 < n) {
+      const double* L2 = A + k2 * lda + k0;
+      if ((err = dgemm(n - k2, n - k2, kb, -1.0, L2, lda, true, L2, lda, true, 1.0, A + k2 * lda + k2, lda, true,
+                       nullptr, sl)) != cudaSuccess)
+        return err;
+      if ((err = cudaEventRecord(h->ev_rest, sl)) != cudaSuccess) return err;
+      rest = true;
+    }
   }
-  return cudaSuccess;
+  // the last rest was waited for before the last panel's update
+  return follow(st, h->ev_panel, sh);
 }
 
 // Same blocked factorisation with the trailing updates on the tensor cores
@@ -1115,6 +1157,8 @@ cudaError_t ensure_chol_streams(gn_handle* h) {
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_hi, cudaStreamNonBlocking, greatest);
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_lo, cudaStreamNonBlocking, middle);
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_g, cudaStreamNonBlocking, least);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_panel, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_rest, cudaEventDisableTiming);
   return e;
 }
 

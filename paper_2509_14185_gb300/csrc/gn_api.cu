@@ -647,6 +647,8 @@ int gn_destroy(gn_handle* h) {
   if (h->st_hi) cudaStreamDestroy(h->st_hi);
   if (h->st_lo) cudaStreamDestroy(h->st_lo);
   if (h->st_g) cudaStreamDestroy(h->st_g);
+  if (h->ev_panel) cudaEventDestroy(h->ev_panel);
+  if (h->ev_rest) cudaEventDestroy(h->ev_rest);
   destroy_side(h);
   free_all(h);
   if (h->tmaps) free(h->tmaps);
@@ -773,7 +775,7 @@ int damped_solve(gn_handle* h, const double* G, const double* g, double* gamma, 
       if (rc) return rc;
       GN_TRY_CUDA(e);
     } else {
-      GN_TRY_CUDA(cholesky_factor(h->A, Pp, Pp, h->Linv, h->flag + 1, h->st));
+      GN_TRY_CUDA(cholesky_factor(h, h->A, Pp, Pp, h->Linv, h->flag + 1));
     }
     int hflag[3] = {0, 0, 0};
     GN_TRY_CUDA(cudaMemcpyAsync(&h->hpin[8], h->flag, 3 * sizeof(int), cudaMemcpyDeviceToHost, h->st));

@@ -145,10 +145,11 @@ struct gn_handle {
   // EMA rank-1 optimiser scratch: u [Pp], J~ Delta [rows], J~ v [rows] (allocated on first use)
   double* ema_ws = nullptr;
   int64_t ema_len = 0;
-  // streams of the split factorisation's look-ahead (created on first use)
+  // streams of the factorisations' look-ahead (created on first use)
   cudaStream_t st_hi = nullptr;   // critical path (highest priority)
   cudaStream_t st_lo = nullptr;   // deferred bulk updates (middle priority)
   cudaStream_t st_g = nullptr;    // Gram chunks of the pipelined step (lowest priority)
+  cudaEvent_t ev_panel = nullptr, ev_rest = nullptr;   // the FP64 factorisation's look-ahead
   // side stream of the wall and normalisation passes (residual and Jacobian modes), with the
   // events that fork it from and join it to the handle's stream
   cudaStream_t st_aux = nullptr;
@@ -280,7 +281,7 @@ cudaError_t hilbert_series_build(const double* y, int64_t n, int M, int order, d
 // Cholesky (FP64, blocked, lower, in place on A row-major) and solves.
 constexpr int kCholNB = 64;
 constexpr int64_t kCholStrip = 4 * kCholNB;   // columns per strip of the split factorisation
-cudaError_t cholesky_factor(double* A, int64_t n, int64_t lda, double* Linv, int* flag, cudaStream_t st);
+cudaError_t cholesky_factor(gn_handle* h, double* A, int64_t n, int64_t lda, double* Linv, int* flag);
 cudaError_t cholesky_solve(const double* A, int64_t n, int64_t lda, const double* Linv, const double* b,
                            double* x, double* tmp, cudaStream_t st);   // tmp: 2n doubles
 // L^T x = y only (the forward half already done, e.g. inside cholesky_factor_split); tmp: n doubles

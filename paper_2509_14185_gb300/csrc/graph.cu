@@ -224,7 +224,7 @@ int capture_solve(gn_handle* h, double* theta, bool marks, const cudaEvent_t* ga
     GN_G_TRY(e);
     GN_G_TRY(cholesky_solve_backward(h->A, Pp, Pp, h->Linv, h->vtmp + Pp, h->delta, h->vtmp, st));
   } else {
-    GN_G_TRY(cholesky_factor(h->A, Pp, Pp, h->Linv, h->flag + 1, st));
+    GN_G_TRY(cholesky_factor(h, h->A, Pp, Pp, h->Linv, h->flag + 1));
     GN_G_TRY(cholesky_solve(h->A, Pp, Pp, h->Linv, h->g, h->delta, h->vtmp, st));
   }
   if (mark(h, marks, 5)) return GN_ERR_CUDA;

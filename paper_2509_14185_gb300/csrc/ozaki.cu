@@ -1166,6 +1166,7 @@ int pretune_gram(gn_handle* h) {
 // largest row block, the CCF Hilbert contraction's operands (SPLIT_ALL) and the split
 // factorisation's workspace and streams (SPLIT_ALL).
 int prepare_for_capture(gn_handle* h) {
+  if (GN_NOTE(ensure_chol_streams(h)) != cudaSuccess) return GN_ERR_CUDA;
   if (h->precision == GN_PREC_FP64) return GN_OK;
   const int S = h->n_slices;
   size_t need = oz_operand_bytes(S, h->Pp, h->jrows) + (size_t)CM_CHUNKS * rup(h->Pp, TM) * 8 + 256 +
@@ -1179,7 +1180,6 @@ int prepare_for_capture(gn_handle* h) {
     }
     const int rc = ensure_chol_ws(h, chol_split_ws_bytes(h->Pp, S));
     if (rc) return rc;
-    if (GN_NOTE(ensure_chol_streams(h)) != cudaSuccess) return GN_ERR_CUDA;
   }
   const int rc = ensure_split_ws(h, need);
   if (rc) return rc;
