@@ -86,7 +86,7 @@ cudaError_t dalloc(T** p, size_t count) {
 }
 
 void free_all(gn_handle* h) {
-  void* ptrs[] = {h->ema_ws, h->wt, h->theta_t, h->r, h->J, h->G, h->A, h->Linv, h->g, h->delta, h->vtmp, h->red,
+  void* ptrs[] = {h->lay_ws, h->ema_ws, h->wt, h->theta_t, h->r, h->J, h->G, h->A, h->Linv, h->g, h->delta, h->vtmp, h->red,
                   h->flag, h->gpart, h->kf, h->dcoef, h->snode, h->gnode, h->Jg, h->ug, h->sU, h->tnode,
                   h->split_ws, h->chol_ws, h->base_int, h->base_wall, h->base_norm, h->base_node, h->fourierW,
                   h->base_inf, h->base_relu, h->kd[0], h->kd[1], h->dd[0], h->dd[1], h->ugd[0], h->ugd[1],
@@ -121,6 +121,15 @@ int64_t edge_row0(const gn_handle* h) { return h->p.n_pts * h->ne + n_drows(h, 1
 
 namespace gn {
 
+static bool takes_layers(const gn_handle* h, const JetArgs& a) { return h->lay_ws && layers_eligible(a); }
+// One point kind on the handle's stream: layer by layer where that pays (layers.cu), else one
+// warp per point.  (The side stream's kinds always take the latter: the layers' scratch is one.)
+static cudaError_t launch_points(gn_handle* h, JetArgs& a, cudaStream_t st) {
+  set_point_range(a);
+  if (takes_layers(h, a)) return launch_layers(a, h->lay_ws, h->lay_ws_bytes, st);
+  return launch_jet(a, st, nullptr);
+}
+
 // Evaluate rows (all kinds) at (theta, lambda) in one mode.  In gradient mode
 // the per-warp partials are reduced into grad (P+1 entries).
 int run_pass(gn_handle* h, const double* theta, double lam, const Pass& ps, double* grad) {
@@ -154,8 +163,7 @@ int run_pass(gn_handle* h, const double* theta, double lam, const Pass& ps, doub
   // (a one-point pass is latency-bound; alone it would add its whole latency); gradient mode
   // accumulates every kind into the same per-warp partials, so it keeps them in order.
   const bool side = ps.mode != MODE_GRADIENT && h->st_aux;
-  auto edge_rows = [&](cudaStream_t sx) -> int {
-    // wall points
+  auto wall_rows = [&](cudaStream_t sx, bool layered) -> int {
     if (h->p.n_bnd > 0) {
       JetArgs b = a;
       b.kind = KIND_WALL;
@@ -172,8 +180,15 @@ int run_pass(gn_handle* h, const double* theta, double lam, const Pass& ps, doub
       b.jrow_lo = ps.jlo;
       b.jrow_hi = ps.jhi;
       b.seed = ps.seed;
-      GN_TRY_CUDA(launch_jet(b, sx, nullptr));
+      // enough wall points for the layered path take it, in order with the interior (one scratch)
+      if (takes_layers(h, b) != layered) return GN_OK;
+      GN_TRY_CUDA(layered ? launch_points(h, b, sx) : launch_jet(b, sx, nullptr));
     }
+    return GN_OK;
+  };
+  auto edge_rows = [&](cudaStream_t sx) -> int {
+    int rc = wall_rows(sx, false);
+    if (rc) return rc;
     // decay rows of the data loss: sqrt(2 c_inf) Phi_A0 at the far points
     if (h->p.n_inf > 0) {
       JetArgs b = a;
@@ -261,7 +276,7 @@ int run_pass(gn_handle* h, const double* theta, double lam, const Pass& ps, doub
     b.jrow_hi = h->Mh;
     b.base = h->staged ? h->base_node : nullptr;
     b.base_ld = 1;
-    GN_TRY_CUDA(launch_jet(b, st, nullptr));
+    GN_TRY_CUDA(launch_points(h, b, st));
     GN_TRY_CUDA(dgemv_n(h->kf, h->Mh, n, h->Mh, h->gnode, h->ug, 0.0, st));
     // the derivative batches' K part, one coefficient of the series in y at a time
     for (int od = 1; od <= 2; od++) {
@@ -292,8 +307,9 @@ int run_pass(gn_handle* h, const double* theta, double lam, const Pass& ps, doub
     b.ug = h->ug;
     b.dcoef = h->dcoef;
     b.sU = h->sU;
-    GN_TRY_CUDA(launch_jet(b, st, nullptr));
+    GN_TRY_CUDA(launch_points(h, b, st));
   }
+  if (int rc = wall_rows(st, true)) return rc;
   // derivative-loss rows (d1, d2)
   for (int od = 1; od <= 2; od++) {
     const int64_t nd = od == 1 ? h->p.n_d1 : h->p.n_d2;
@@ -597,6 +613,14 @@ int gn_init(const gn_problem* p, void* cuda_stream, gn_handle** out) {
     free_all(h);
     delete h;
     return GN_ERR_OOM;
+  }
+  // the layered passes' scratch; without it they run one warp per point
+  int64_t most = p->n_pts > h->Mh ? p->n_pts : h->Mh;
+  if (p->n_bnd > most) most = p->n_bnd;
+  h->lay_ws_bytes = layers_ws_bytes(net, h->d, h->nf, h->ne, most);
+  if (h->lay_ws_bytes > 0 && cudaMalloc(&h->lay_ws, h->lay_ws_bytes) != cudaSuccess) {
+    cudaGetLastError();
+    h->lay_ws = nullptr;
   }
   cudaError_t e = cudaMemsetAsync(h->flag, 0, 4 * sizeof(int), h->st);
   if (e == cudaSuccess && net.fourier) {

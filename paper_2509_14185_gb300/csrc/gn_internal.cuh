@@ -67,6 +67,7 @@ struct JetArgs {
   double lam;
   const double* lamp;    // device copy of lambda (null: use lam); graph-captured steps read it here
   int64_t n;             // points of this kind
+  int64_t pt0, pt1;      // points evaluated, [pt0, pt1) of the n (set_point_range)
   const double* y;       // SoA [d][ystride]
   int64_t ystride;
   const double* rho;     // interior weights (may be null)
@@ -142,6 +143,9 @@ struct gn_handle {
   void* split_ws;
   size_t split_ws_bytes;
   void* tmaps;            // host copies of TMA descriptors
+  // scratch of the layered passes (null: too few points, or no memory to spare for it)
+  void* lay_ws;
+  size_t lay_ws_bytes;
   // EMA rank-1 optimiser scratch: u [Pp], J~ Delta [rows], J~ v [rows] (allocated on first use)
   double* ema_ws = nullptr;
   int64_t ema_len = 0;
@@ -219,7 +223,13 @@ void graph_release(gn_handle* h);
 
 // ---- launchers (host functions implemented in the .cu files) -----------
 cudaError_t launch_transpose_weights(const NetDesc& net, const double* theta, double* wt, cudaStream_t st);
+void set_point_range(JetArgs& a);   // the points that own rows of the launch
 cudaError_t launch_jet(const JetArgs& a, cudaStream_t st, int64_t* warps_used);
+// many points at once, layer by layer (layers.cu); ws: layers_ws_bytes of the network and its
+// largest point set (0: never eligible)
+bool layers_eligible(const JetArgs& a);
+size_t layers_ws_bytes(const NetDesc& net, int d, int nf, int ne, int64_t npt);
+cudaError_t launch_layers(const JetArgs& a, void* ws, size_t ws_bytes, cudaStream_t st);
 // derivative-loss rows of order ord (1: d1, 2: d2) at the a.n points (djet.cu); a.row0 is the
 // first row, a.wscale sqrt(2 c_d / (N_d N_E d^ord)).  CCF: a.ug / a.dcoef hold the K part's
 // and D's Taylor coefficients in y ([m][n], m <= order_y), a.sU receives d row / d U_m ([m][n],

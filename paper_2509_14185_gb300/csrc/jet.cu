@@ -27,9 +27,7 @@
 //     sum_c abar_c[o] h_c[i] are written as consecutive addresses by
 //     consecutive lanes (coalesced J row stores), or accumulated into a
 //     per-warp partial gradient (adjoint mode).
-#include <cmath>
-
-#include "gn_internal.cuh"
+#include "chain.cuh"
 
 namespace gn {
 namespace {
@@ -37,151 +35,6 @@ namespace {
 // Grid cap: two resident blocks per SM keep the FP64 pipe busy (the kernel is
 // FP64-bound); it also bounds the per-warp partial-gradient buffer.
 constexpr int64_t kJetMaxBlocks = 152 * 2;
-
-struct Dl {
-  double v, d;
-};
-__device__ __forceinline__ Dl operator+(Dl a, Dl b) { return {a.v + b.v, a.d + b.d}; }
-__device__ __forceinline__ Dl operator-(Dl a, Dl b) { return {a.v - b.v, a.d - b.d}; }
-__device__ __forceinline__ Dl operator-(Dl a) { return {-a.v, -a.d}; }
-__device__ __forceinline__ Dl operator*(Dl a, Dl b) { return {a.v * b.v, fma(a.v, b.d, a.d * b.v)}; }
-__device__ __forceinline__ Dl operator*(double s, Dl a) { return {s * a.v, s * a.d}; }
-__device__ __forceinline__ Dl operator+(double s, Dl a) { return {s + a.v, a.d}; }
-__device__ __forceinline__ Dl dconst(double v) { return {v, 0.0}; }
-// u^e for a constant base u > 0 and a dual exponent e.
-__device__ __forceinline__ Dl pow_cb(double u, Dl e) {
-  const double lu = log(u);
-  const double p = exp(e.v * lu);
-  return {p, p * lu * e.d};
-}
-
-template <int EQ> struct Eq;
-template <> struct Eq<GN_BURGERS> { static constexpr int D = 1, NF = 1, NE = 1; };
-template <> struct Eq<GN_CCF> { static constexpr int D = 1, NF = 1, NE = 1; };
-template <> struct Eq<GN_IPM> { static constexpr int D = 2, NF = 2, NE = 2; };
-template <> struct Eq<GN_BOUSSINESQ> { static constexpr int D = 2, NF = 3, NE = 3; };
-
-// Network-input jet components.  1D: (v, z, zz).  2D: (v, q, b, qq, qb, bb,
-// qqq, qqb, qbb).  The reverse pass uses the first C_R of them.
-template <int D> struct JT;
-template <> struct JT<1> { static constexpr int CR = 2, CF = 3; };
-template <> struct JT<2> { static constexpr int CR = 6, CF = 9; };
-
-// Component reached by one more derivative along q (used for d/dlambda,
-// since lambda enters the network only through q).
-template <int D> __device__ __forceinline__ int q_shift(int c);
-template <> __device__ __forceinline__ int q_shift<1>(int c) { return c + 1; }
-template <> __device__ __forceinline__ int q_shift<2>(int c) {
-  // v->q, q->qq, b->qb, qq->qqq, qb->qqb, bb->qbb
-  const int m[6] = {1, 3, 4, 6, 7, 8};
-  return m[c];
-}
-
-// y-jet of dual numbers: value, first derivatives, second derivatives
-// (1D: h[0] = d11; 2D: h[0] = d11, h[1] = d12, h[2] = d22).
-template <int D> struct YJ {
-  Dl v;
-  Dl g[D];
-  Dl h[D == 1 ? 1 : 3];
-};
-template <int D> __device__ __forceinline__ int hix(int i, int j) { return D == 1 ? 0 : i + j; }
-
-template <int D> __device__ __forceinline__ YJ<D> ymul(const YJ<D>& a, const YJ<D>& b) {
-  YJ<D> c;
-  c.v = a.v * b.v;
-#pragma unroll
-  for (int i = 0; i < D; i++) c.g[i] = a.g[i] * b.v + a.v * b.g[i];
-#pragma unroll
-  for (int i = 0; i < D; i++)
-#pragma unroll
-    for (int j = i; j < D; j++) {
-      const int k = hix<D>(i, j);
-      c.h[k] = a.h[k] * b.v + a.g[i] * b.g[j] + a.g[j] * b.g[i] + a.v * b.h[k];
-    }
-  return c;
-}
-
-// Envelope y1^m * u^e (u = 1 + |y|^2) as a y-jet; e is a dual number.
-//   (u^e)_i = 2 e y_i u^e / u,  (u^e)_ij = 2 e u^e / u (delta_ij + 2 (e-1) y_i y_j / u).
-template <int D> __device__ YJ<D> envelope(const double* y, double u, int m, Dl e) {
-  const Dl W = pow_cb(u, e);
-  const double iu = 1.0 / u;
-  const Dl c1 = (2.0 * iu) * (e * W);  // 2 e W / u
-  YJ<D> Wj;
-  Wj.v = W;
-#pragma unroll
-  for (int i = 0; i < D; i++) Wj.g[i] = y[i] * c1;
-  const Dl em1 = e + dconst(-1.0);
-#pragma unroll
-  for (int i = 0; i < D; i++)
-#pragma unroll
-    for (int j = i; j < D; j++) {
-      const Dl inner = dconst(i == j ? 1.0 : 0.0) + (2.0 * y[i] * y[j] * iu) * em1;
-      Wj.h[hix<D>(i, j)] = c1 * inner;
-    }
-  if (m == 0) return Wj;
-  YJ<D> Y;
-  const double y1 = y[0];
-  Y.v = dconst(m == 1 ? y1 : y1 * y1);
-#pragma unroll
-  for (int i = 0; i < D; i++) Y.g[i] = dconst(0.0);
-  Y.g[0] = dconst(m == 1 ? 1.0 : 2.0 * y1);
-#pragma unroll
-  for (int k = 0; k < (D == 1 ? 1 : 3); k++) Y.h[k] = dconst(0.0);
-  Y.h[0] = dconst(m == 1 ? 0.0 : 2.0);
-  return ymul<D>(Y, Wj);
-}
-
-// Exponential output map on one field's jet components a[0 .. CF) (value, q, (b,) the second
-// orders, the q-direction third orders the lambda column needs): N = exp(a) by the chain rule,
-// every component exp(a_v) times the complete Bell polynomial of the a-derivatives.
-template <int D, int CF>
-__device__ __forceinline__ void exp_jet(const double* a, double* N) {
-  const double E = exp(a[0]);
-  N[0] = E;
-  if constexpr (D == 1) {
-    N[1] = E * a[1];
-    if constexpr (CF > 2) N[2] = E * (a[2] + a[1] * a[1]);
-  } else {
-    const double q = a[1], b = a[2];
-    N[1] = E * q;
-    N[2] = E * b;
-    N[3] = E * (a[3] + q * q);
-    N[4] = E * (a[4] + q * b);
-    N[5] = E * (a[5] + b * b);
-    if constexpr (CF > 6) {
-      N[6] = E * (a[6] + 3.0 * q * a[3] + q * q * q);
-      N[7] = E * (a[7] + b * a[3] + 2.0 * q * a[4] + q * q * b);
-      N[8] = E * (a[8] + q * a[5] + 2.0 * b * a[4] + q * b * b);
-    }
-  }
-}
-
-// Its adjoint on the components the reverse pass carries (c < C_R): nb holds dN-bar on entry
-// and the pre-activation adjoints a-bar_c = sum_k N-bar_k dN_k / da_c on exit.
-template <int D>
-__device__ __forceinline__ void exp_jet_adjoint(const double* a, double* nb) {
-  const double E = exp(a[0]);
-  if constexpr (D == 1) {
-    const double a0 = nb[0] * E + nb[1] * (E * a[1]);
-    nb[1] = nb[1] * E;
-    nb[0] = a0;
-  } else {
-    const double q = a[1], b = a[2];
-    const double N[6] = {E, E * q, E * b, E * (a[3] + q * q), E * (a[4] + q * b), E * (a[5] + b * b)};
-    double s = 0.0;
-#pragma unroll
-    for (int c = 0; c < 6; c++) s = fma(nb[c], N[c], s);
-    const double a1 = E * (nb[1] + 2.0 * q * nb[3] + b * nb[4]);
-    const double a2 = E * (nb[2] + q * nb[4] + 2.0 * b * nb[5]);
-    nb[0] = s;
-    nb[1] = a1;
-    nb[2] = a2;
-    nb[3] *= E;
-    nb[4] *= E;
-    nb[5] *= E;
-  }
-}
 
 // Per-warp shared-memory layout (doubles).  H[j][c][ldw] for c < C_R: j = 0 network
 // input, j = 1..L-1 outputs of hidden layers (the reverse pass reads them); the forward-only
@@ -232,7 +85,7 @@ __global__ void __launch_bounds__(256, Eq<EQ>::D == 1 ? 2 : 1) jet_kernel(const 
   const int K = 1 + NF * CR;                  // tangent directions in use
   const int dir = (lane < K) ? lane : 0;      // this lane's direction
 
-  for (int64_t pt = gw; pt < A.n; pt += nw) {
+  for (int64_t pt = A.pt0 + gw; pt < A.pt1; pt += nw) {
     double y[D];
 #pragma unroll
     for (int k = 0; k < D; k++) y[k] = A.y[(int64_t)k * A.ystride + pt];
@@ -352,68 +205,9 @@ __global__ void __launch_bounds__(256, Eq<EQ>::D == 1 ? 2 : 1) jet_kernel(const 
         }
         nn[f][c] = {NN[f * CF + c], dv};
       }
-    // q jets: q_i = -a y_i q / u ; q_ij = -a q / u (delta_ij - (a+2) y_i y_j / u)
-    const double iu = 1.0 / u;
-    Dl qg[D], qh[D == 1 ? 1 : 3];
-    const Dl aq_u = (-iu) * (a * q);
-#pragma unroll
-    for (int i = 0; i < D; i++) qg[i] = y[i] * aq_u;
-#pragma unroll
-    for (int i = 0; i < D; i++)
-#pragma unroll
-      for (int j = i; j < D; j++)
-        qh[hix<D>(i, j)] = aq_u * (dconst(i == j ? 1.0 : 0.0) + (-y[i] * y[j] * iu) * (a + dconst(2.0)));
-    // beta jets (2D): beta_1 = -y1 y2 u^-3/2, beta_2 = (1+y1^2) u^-3/2,
-    // beta_11 = y2 (3 y1^2 - u) u^-5/2, beta_12 = y1 (3 y2^2 - u) u^-5/2,
-    // beta_22 = -3 y2 (1 + y1^2) u^-5/2
-    double bg[2] = {0.0, 0.0}, bh[3] = {0.0, 0.0, 0.0};
-    if (D == 2) {
-      const double s3 = iu / sqrt(u), s5 = s3 * iu;
-      bg[0] = -y[0] * y[1] * s3;
-      bg[1] = (1.0 + y[0] * y[0]) * s3;
-      bh[0] = y[1] * (3.0 * y[0] * y[0] - u) * s5;
-      bh[1] = y[0] * (3.0 * y[1] * y[1] - u) * s5;
-      bh[2] = -3.0 * y[1] * (1.0 + y[0] * y[0]) * s5;
-    }
     const Dl lamd = {lam, (dir == 0 && MODE != MODE_RESIDUAL) ? 1.0 : 0.0};
-    // fields F_f = E_f * N_f
     YJ<D> F[NF];
-#pragma unroll
-    for (int f = 0; f < NF; f++) {
-      YJ<D> N;
-      N.v = nn[f][0];
-      if (D == 1) {
-        N.g[0] = nn[f][1] * qg[0];
-        N.h[0] = dconst(0.0);  // not used by the 1D residuals
-      } else {
-#pragma unroll
-        for (int i = 0; i < D; i++) N.g[i] = nn[f][1] * qg[i] + bg[i] * nn[f][2];
-#pragma unroll
-        for (int i = 0; i < D; i++)
-#pragma unroll
-          for (int j = i; j < D; j++) {
-            const int k = hix<D>(i, j);
-            N.h[k] = nn[f][3] * (qg[i] * qg[j]) + nn[f][4] * (bg[j] * qg[i] + bg[i] * qg[j]) +
-                     (bg[i] * bg[j]) * nn[f][5] + nn[f][1] * qh[k] + bh[k] * nn[f][2];
-          }
-      }
-      // exponent k_f(lambda) and prefactor (y1^m, extra power of u)
-      Dl kf;
-      int m;
-      double e0;
-      if (EQ == GN_BURGERS) { kf = lamd; m = 1; e0 = -0.5; }
-      else if (EQ == GN_CCF) { kf = lamd; m = 2; e0 = -1.0; }
-      else if (EQ == GN_IPM) {
-        if (f == 0) { kf = lamd; m = 0; e0 = 0.0; }
-        else { kf = dconst(1.0) + 2.0 * lamd; m = 1; e0 = -0.5; }
-      } else {
-        if (f == 0) { kf = dconst(-1.0); m = 1; e0 = -0.5; }
-        else if (f == 1) { kf = lamd + dconst(-1.0); m = 0; e0 = 0.0; }
-        else { kf = dconst(1.0) + 2.0 * lamd; m = 1; e0 = -0.5; }
-      }
-      const Dl e = dconst(e0) + 0.5 * (kf * a);
-      F[f] = ymul<D>(envelope<D>(y, u, m, e), N);
-    }
+    field_jets<EQ>(y, u, a, q, lamd, beta, nn, F);
     constexpr int NJ = 1 + D + (D == 1 ? 1 : 3);   // probe values per field
 
     if (kind == KIND_PROBE) {
@@ -438,79 +232,9 @@ __global__ void __launch_bounds__(256, Eq<EQ>::D == 1 ? 2 : 1) jet_kernel(const 
       continue;
     }
 
-    // stage 2: Phi = Phi_1 + eps Phi_2, Phi_1 a constant (its jets precomputed at this point)
-    if (A.base && kind != KIND_NODE) {
-      const double* b = A.base + pt * A.base_ld;
-      const double ep = A.eps;
-#pragma unroll
-      for (int f = 0; f < NF; f++) {
-        F[f].v = Dl{b[f * NJ] + ep * F[f].v.v, ep * F[f].v.d};
-#pragma unroll
-        for (int i = 0; i < D; i++) F[f].g[i] = Dl{b[f * NJ + 1 + i] + ep * F[f].g[i].v, ep * F[f].g[i].d};
-#pragma unroll
-        for (int k = 0; k < (D == 1 ? 1 : 3); k++)
-          F[f].h[k] = Dl{b[f * NJ + 1 + D + k] + ep * F[f].h[k].v, ep * F[f].h[k].d};
-      }
-    }
-
-    // residuals (or the single value of a wall/node/norm row)
     Dl R[NE];
-    double sUv = 0.0;
-    const Dl opl = dconst(1.0) + lamd;
-    if (kind == KIND_INTERIOR) {
-      if (EQ == GN_BURGERS) {
-        const YJ<D>& U = F[0];
-        R[0] = (-1.0) * (lamd * U.v) + (y[0] * opl + U.v) * U.g[0];
-      } else if (EQ == GN_CCF) {
-        // U = sum_j K_ij g_j + D_i g(y_i); the K part's d/dlambda is added by
-        // the Hilbert contraction (it carries the lambda column of J_g).
-        const YJ<D> Eg = envelope<D>(y, u, 1, dconst(-1.0) + 0.5 * (lamd * a));
-        Dl gi = Eg.v * nn[0][0];
-        if (A.base) gi = Dl{A.base[pt * A.base_ld + NF * NJ] + A.eps * gi.v, A.eps * gi.d};
-        const Dl Uv = dconst(A.ug[pt]) + A.dcoef[pt] * gi;
-        const YJ<D>& T = F[0];
-        R[0] = (-1.0) * (lamd * T.v) + (y[0] * opl + Uv) * T.g[0];
-        sUv = T.g[0].v;
-      } else if (EQ == GN_IPM) {
-        const YJ<D>& P = F[0];
-        const YJ<D>& S = F[1];
-        const Dl V1 = y[0] * opl + S.g[1];
-        const Dl V2 = y[D - 1] * opl + (-S.g[0]);
-        R[0] = (-1.0) * (lamd * P.v) + V1 * P.g[0] + V2 * P.g[D - 1];
-        R[NE > 1 ? 1 : 0] = S.h[0] + S.h[D == 1 ? 0 : 2] - P.g[0];
-      } else {
-        const YJ<D>& Om = F[0];
-        const YJ<D>& Th = F[NF > 1 ? 1 : 0];
-        const YJ<D>& S = F[NF - 1];
-        const Dl V1 = y[0] * opl + S.g[D - 1];
-        const Dl V2 = y[D - 1] * opl + (-S.g[0]);
-        R[0] = Om.v + V1 * Om.g[0] + V2 * Om.g[D - 1] - Th.g[0];
-        R[NE > 1 ? 1 : 0] = (dconst(1.0) - lamd) * Th.v + V1 * Th.g[0] + V2 * Th.g[D - 1];
-        R[NE > 2 ? 2 : 0] = S.h[0] + S.h[D == 1 ? 0 : 2] + Om.v;
-      }
-    } else if (kind == KIND_WALL) {
-      R[0] = F[NF - 1].v;
-    } else if (kind == KIND_NORM || kind == KIND_INF || kind == KIND_RELU) {
-      // normalisation: Phi_A0 or its d/dy1 minus the target; decay: Phi_A0 itself; bound:
-      // relu(s (Phi_A0 - b)), zero (with a zero derivative) while the bound holds
-      Dl val = F[0].v, dy1 = F[0].g[0];
-#pragma unroll
-      for (int f = 1; f < NF; f++)   // constant register indices only
-        if (f == A.nfield) {
-          val = F[f].v;
-          dy1 = F[f].g[0];
-        }
-      R[0] = (kind == KIND_NORM && A.nderiv) ? dy1 : val;
-      R[0].v -= A.c_norm;
-      if (kind == KIND_RELU) {
-        R[0] = (double)A.rsign * R[0];
-        if (!(R[0].v > 0.0)) R[0] = Dl{0.0, 0.0};
-      }
-    } else {  // KIND_NODE (CCF): g = y/u * NN * q^{-lambda}
-      const YJ<D> Eg = envelope<D>(y, u, 1, dconst(-1.0) + 0.5 * (lamd * a));
-      R[0] = Eg.v * nn[0][0];
-      if (A.base) R[0] = Dl{A.base[pt] + A.eps * R[0].v, A.eps * R[0].d};
-    }
+    double sUv;
+    residual_rows<EQ>(A, kind, pt, y, u, a, lamd, nn, F, R, sUv);
 
     // ---- 4. rows ------------------------------------------------------------
     double w = A.wscale;
@@ -687,7 +411,8 @@ cudaError_t launch_eq(const JetArgs& a, cudaStream_t st, int64_t* warps_used) {
     return ok ? v : 152;
   }();
   int wpb = 8;
-  const int64_t spread = (a.n + sms - 1) / sms;
+  const int64_t npt = a.pt1 - a.pt0;
+  const int64_t spread = (npt + sms - 1) / sms;
   if (spread < wpb) wpb = spread < 1 ? 1 : (int)spread;
   while (wpb > 1 && per_warp * wpb > kSmemCap) wpb--;
   if (per_warp > kSmemCap) return cudaErrorInvalidValue;
@@ -697,12 +422,12 @@ cudaError_t launch_eq(const JetArgs& a, cudaStream_t st, int64_t* warps_used) {
   cudaError_t err = cudaFuncSetAttribute(jet_kernel<EQ, MODE, XO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSmemCap);
   if (err != cudaSuccess) return err;
-  int64_t blocks = (a.n + wpb - 1) / wpb;
+  int64_t blocks = (npt + wpb - 1) / wpb;
   const int64_t cap = kJetMaxBlocks;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
   if (warps_used) *warps_used = blocks * wpb;
-  if (a.n == 0) return cudaSuccess;
+  if (npt <= 0) return cudaSuccess;
   jet_kernel<EQ, MODE, XO><<<(unsigned)blocks, wpb * 32, smem, st>>>(a);
   count_launch();
   return cudaGetLastError();
@@ -724,7 +449,23 @@ cudaError_t launch_mode(const JetArgs& a, cudaStream_t st, int64_t* w) {
 
 }  // namespace
 
-cudaError_t launch_jet(const JetArgs& a, cudaStream_t st, int64_t* warps_used) {
+void set_point_range(JetArgs& a) {
+  a.pt0 = 0;
+  a.pt1 = a.n;
+  if (a.mode != MODE_JACOBIAN) return;
+  // A row block evaluates the points that own one of its rows, and no others (the rows r of the
+  // rest come with their own blocks): a quarter of IPM's rows (16384 points of 65536, 64 x 4)
+  // took 29.2 ms with every point's forward pass, the whole Jacobian 62.
+  const int64_t nrow = a.kind == KIND_INTERIOR ? (a.eq == GN_IPM ? 2 : a.eq == GN_BOUSSINESQ ? 3 : 1) : 1;
+  const int64_t lo = a.jrow_lo - a.row0, hi = a.jrow_hi - a.row0;   // rows of this kind, from its first
+  a.pt0 = lo > 0 ? lo / nrow : 0;
+  a.pt1 = hi > 0 ? (hi + nrow - 1) / nrow : 0;
+  if (a.pt1 > a.n) a.pt1 = a.n;
+}
+
+cudaError_t launch_jet(const JetArgs& args, cudaStream_t st, int64_t* warps_used) {
+  JetArgs a = args;
+  set_point_range(a);
   switch (a.eq) {
     case GN_BURGERS: return launch_mode<GN_BURGERS>(a, st, warps_used);
     case GN_CCF: return launch_mode<GN_CCF>(a, st, warps_used);

@@ -1,0 +1,907 @@
+// Layered evaluation of many points: the network's hidden layers as split GEMMs on the tcgen05
+// tensor cores, the rest pointwise (Methods, "Solution Modeling", "Training Loss" and
+// "Second-order Optimizer": the same rows, Jacobian rows and adjoint as jet.cu).
+//
+// jet.cu carries one point per warp and spends nearly all its time in the FP64 products of the
+// hidden layers (GB300 runs one FP64 warp instruction per 17 clocks and SM).  Here the jets of a
+// chunk of points pass through each hidden layer together, as the rows of a (points x components)
+// x width product, and only the pointwise work stays FP64:
+//
+//   lay_inputs    q, beta of the points; the hidden weights cut into slices
+//   lay_gemm      forward, per hidden layer j: H_j = tanh jets of Z_j, Z_{j+1} = W_j H_j + b_j
+//   lay_last      H_{L-1} and the network outputs NN
+//   lay_chain     one thread per point and tangent direction: residuals, the lambda column and the
+//                 reverse-pass seeds (chain.cuh, the chain jet.cu evaluates per warp)
+//   lay_gemm      reverse, per hidden layer: abar_{j+1} = Hbar_{j+1} through the tanh jets,
+//                 Hbar_j = W_j^T abar_{j+1}
+//   lay_entries   the Jacobian rows sum_c abar_c[o] h_c[i]
+//
+// Precision of the products: every row of either operand is scaled by a power of two and rounded to
+// a 55-bit integer (its largest element keeps two bits more than FP64's own 53), written as 7
+// balanced base-256 digits (exact in BF16).  The 28 digit pairs of the seven leading levels are summed
+// per level in FP32 accumulators, exactly (at most 7 * 64 products below 2^14 each: < 2^23), and the levels are
+// combined in 64-bit integers and rounded once.  What is dropped lies 2^-55 below the largest products, under
+// the rounding of an FP64 sum of 64 terms.
+#include <cmath>
+#include <cstring>
+
+#include "chain.cuh"
+#include "tc.cuh"
+
+namespace gn {
+namespace {
+
+constexpr int kLayS = 7;                           // digits per value
+constexpr int kLayW = 64;                          // widest hidden layer
+constexpr int kLayThreads = 512;
+constexpr int kLayASlice = 2 * 128 * 64;           // one digit of the A tile: two 32-wide K stages
+constexpr int kLayWSlice = 2 * kLayW * 64;         // one digit of the weights
+constexpr int kLayA = kLayS * kLayASlice;          // 112 KB
+constexpr size_t kLaySmem = 1024 + kLayA + kLayS * kLayWSlice + 1024;
+constexpr int kLayBad = 0x3fffffff;                // exponent of a row with a non-finite element
+
+struct LayArgs {
+  int64_t items;            // points (forward) or points x rows (reverse)
+  int nr;                   // rows per point
+  int K, N;                 // width of the producing and of the resulting layer
+  int nf, cz;               // network fields; components per point in zin
+  const double* qb;         // [point][2]: q, beta
+  const double* W0;         // first layer (K x d) and its bias, for the analytic Z_1
+  const double* b0;
+  const double* zin;        // [point][cz][K]: preactivation jets of the producing layer, without its bias
+  const double* bias;       // forward: of the producing layer
+  double* hout;             // forward: [point][CR][K] activation jets (null: not kept)
+  const double* hin;        // reverse: the same, of the layer the adjoint passes
+  const double* seeds;      // reverse from the outputs: [item][nf][CR]
+  const double* Wlast;      // [nf][K]
+  const double* hbar;       // reverse: [item][CR][K]
+  double* abar;             // reverse out: [item][CR][K]
+  double* out;              // [item][C][N]
+  const unsigned char* wsl; // weight digits, kLayS x 64 x 64 BF16
+  const int* we;            // weight exponents [64]
+  int* flag;
+  unsigned long long wait_ns;
+};
+
+// tanh jets at one neuron: h[0..C) from the preactivation components z[0..C)
+template <int D, int C>
+__device__ __forceinline__ void tanh_jet(const double* z, double* h) {
+  const double t = tanh(z[0]);
+  const double t1 = 1.0 - t * t;
+  h[0] = t;
+  if constexpr (D == 1) {
+    h[1] = t1 * z[1];
+    if constexpr (C > 2) {
+      const double t2 = -2.0 * t * t1;
+      h[2] = t2 * z[1] * z[1] + t1 * z[2];
+    }
+  } else {
+    const double t2 = -2.0 * t * t1;
+    const double q = z[1], b = z[2];
+    h[1] = t1 * q;
+    h[2] = t1 * b;
+    const double t2q = t2 * q, t2b = t2 * b;
+    h[3] = t2q * q + t1 * z[3];
+    h[4] = t2q * b + t1 * z[4];
+    h[5] = t2b * b + t1 * z[5];
+    if constexpr (C > 6) {
+      const double t3 = -2.0 * t1 * t1 - 2.0 * t * t2;
+      const double t3qq = t3 * q * q;
+      h[6] = t3qq * q + 3.0 * t2q * z[3] + t1 * z[6];
+      h[7] = t3qq * b + t2 * (2.0 * q * z[4] + b * z[3]) + t1 * z[7];
+      h[8] = t3 * q * b * b + t2 * (2.0 * b * z[4] + q * z[5]) + t1 * z[8];
+    }
+  }
+}
+
+// adjoint of the tanh jets at one neuron: g = Hbar on entry, abar on exit; t = tanh, z[1..CR) the
+// preactivation derivatives
+template <int D>
+__device__ __forceinline__ void tanh_jet_adjoint(double t, const double* z, double* g) {
+  const double t1 = 1.0 - t * t, t2 = -2.0 * t * t1;
+  if constexpr (D == 1) {
+    g[0] = g[0] * t1 + g[1] * t2 * z[1];
+    g[1] = g[1] * t1;
+  } else {
+    const double t3 = -2.0 * t1 * t1 - 2.0 * t * t2;
+    const double q = z[1], b = z[2];
+    const double g3q = g[3] * q, g4b = g[4] * b, g4q = g[4] * q, g5b = g[5] * b;
+    g[0] = g[0] * t1 + t2 * (g[1] * q + g[2] * b + g[3] * z[3] + g[4] * z[4] + g[5] * z[5]) +
+           t3 * (g3q * q + g4q * b + g5b * b);
+    g[1] = g[1] * t1 + t2 * (2.0 * g3q + g4b);
+    g[2] = g[2] * t1 + t2 * (g4q + 2.0 * g5b);
+    g[3] *= t1;
+    g[4] *= t1;
+    g[5] *= t1;
+  }
+}
+
+// preactivation jets of the first hidden layer: linear in (q, beta)
+template <int D, int C>
+__device__ __forceinline__ void first_layer(const double* W0, const double* b0, int o, double q, double beta,
+                                            double* z) {
+#pragma unroll
+  for (int c = 1; c < C; c++) z[c] = 0.0;
+  if constexpr (D == 1) {
+    const double w = W0[o];
+    z[0] = fma(w, q, b0[o]);
+    z[1] = w;
+  } else {
+    const double w = W0[2 * o], v = W0[2 * o + 1];
+    z[0] = fma(v, beta, fma(w, q, b0[o]));
+    z[1] = w;
+    z[2] = v;
+  }
+}
+
+__device__ __forceinline__ unsigned abs_hi(double x) {
+  return (unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu;
+}
+// e with 2^e > every |x| whose largest high word is m (kLayBad: one of them is not finite)
+__device__ __forceinline__ int row_exponent(unsigned m) {
+  const int ex = (int)(m >> 20);
+  return ex == 0x7ff ? kLayBad : (ex > 0 ? ex : 1) - 1022;
+}
+// x 2^(55 - e) to the nearest integer plus the digits' bias: bytes 0..5 are then digits 6..1 plus
+// 128 and the rest, shifted right arithmetically, is digit 0.
+__device__ __forceinline__ long long biased_digits(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+  if (ex > 0) m |= 1ull << 52;
+  const int sh = (ex > 0 ? ex : 1) - 1020 - e;   // <= 2
+  unsigned long long v;
+  if (sh >= 0) v = m << sh;
+  else v = sh < -54 ? 0ull : (m + (1ull << (-sh - 1))) >> -sh;
+  return ((b >> 63) ? -(long long)v : (long long)v) + 0x808080808080ll;
+}
+// digit q of a biased value as BF16 bits (an integer of at most 8 significant bits: the upper half
+// of its FP32 form)
+__device__ __forceinline__ unsigned short digit_bf16(long long u, int q) {
+  const unsigned lo = (unsigned)u, hi = (unsigned)((unsigned long long)u >> 32);
+  float f;
+  if (q == 0) f = (float)((int)hi >> 16);
+  else {
+    const int byte = 6 - q;   // 0..5
+    f = __uint_as_float(__byte_perm(byte < 4 ? lo : hi, 0x4B000000u, 0x7540 + (byte & 3))) - 8388736.0f;
+  }
+  return (unsigned short)(__float_as_uint(f) >> 16);
+}
+// byte offset of element (row, k) in a K-major operand tile with the 64-byte swizzle, `rows` rows
+__device__ __forceinline__ int swz(int row, int k, int rows) {
+  return (k >> 5) * rows * 64 + row * 64 + ((((k & 31) >> 3) ^ ((row >> 1) & 3)) << 4) + (k & 7) * 2;
+}
+
+// T 2^k rounded to nearest even, by integer operations (an I2F and a multiply would take two slots of the FP64
+// pipe per element); FP64 where the result leaves the normal range
+__device__ __forceinline__ double scaled_int(long long T, int k) {
+  if (T == 0) return 0.0;
+  const unsigned long long m = T < 0 ? (unsigned long long)-T : (unsigned long long)T;
+  const int lz = __clzll((long long)m);
+  const int e = 1023 + 63 - lz + k;
+  if (e <= 0 || e >= 2046) return ldexp((double)T, k);
+  const unsigned long long n = m << lz;                       // leading one at bit 63
+  const unsigned long long rem = n & 0x7ff;
+  unsigned long long r = ((unsigned long long)(e - 1) << 52) + (n >> 11);   // the leading one carries into e
+  if (rem > 0x400 || (rem == 0x400 && (r & 1))) r++;
+  return __longlong_as_double((long long)(r | ((unsigned long long)T & 0x8000000000000000ull)));
+}
+
+// ---- inputs and weight slices --------------------------------------------------------------------
+struct LayPrep {
+  const double* y;
+  int64_t ystride, pt0, npt;
+  double lam;
+  const double* lamp;
+  double* qb;
+  const double* theta;
+  NetDesc net;
+  unsigned char* wsl;       // [(layer - 1) * 2 + direction][kLayS][64][64] BF16
+  int* we;                  // [...][64]
+  int pt_blocks;
+};
+template <int D>
+__global__ void __launch_bounds__(256) lay_inputs(const LayPrep p) {
+  if ((int)blockIdx.x < p.pt_blocks) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= p.npt) return;
+    const double lam = p.lamp ? *p.lamp : p.lam;
+    double u = 1.0, y1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < D; k++) {
+      const double v = p.y[(int64_t)k * p.ystride + p.pt0 + i];
+      u = fma(v, v, u);
+      if (k == 1) y1 = v;
+    }
+    const Dl a = {1.0 / (1.0 + lam), 0.0};
+    p.qb[2 * i] = pow_cb(u, -0.5 * a).v;
+    p.qb[2 * i + 1] = D == 2 ? y1 / sqrt(u) : 0.0;
+    return;
+  }
+  // weights: one warp per operand row.  Forward operand of layer l: row o is W_l[o][.]; reverse:
+  // row i is W_l[.][i].
+  const int w = ((int)blockIdx.x - p.pt_blocks) * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int op = w / kLayW, row = w % kLayW, l = 1 + op / 2, rev = op & 1;
+  if (l > p.net.L - 2) return;
+  const int in = p.net.w[l], out = p.net.w[l + 1];
+  const double* W = p.theta + p.net.offW[l];
+  double x[2];
+  unsigned m = 0;
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    const int k = lane + 32 * q;
+    const int o = rev ? k : row, i = rev ? row : k;
+    x[q] = (o < out && i < in) ? W[(int64_t)o * in + i] : 0.0;
+    const unsigned h = abs_hi(x[q]);
+    m = h > m ? h : m;
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  const int e = row_exponent(m);
+  if (lane == 0) p.we[op * kLayW + row] = e;
+  unsigned short* dst = reinterpret_cast<unsigned short*>(p.wsl) + (size_t)op * kLayS * kLayW * kLayW + row * kLayW;
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    const long long u = biased_digits(x[q], e == kLayBad ? 0 : e);
+#pragma unroll
+    for (int s = 0; s < kLayS; s++) dst[s * kLayW * kLayW + lane + 32 * q] = digit_bf16(u, s);
+  }
+}
+
+// ---- one hidden layer ------------------------------------------------------------------------------
+enum LayKind : int { LAY_FWD_FIRST = 0, LAY_FWD = 1, LAY_REV_LAST = 2, LAY_REV = 3 };
+
+// One CTA per SM, persistent over tiles of 128 rows (128 / C items of C components).  Its 16 warps
+// first produce the tile's A operand, one item per warp: FP64 jets through tanh (or its adjoint),
+// the rows' exponents, their digits into shared memory in the layout the MMA reads.  One thread
+// then issues the 28 digit-pair products into seven tensor-memory accumulators of 64 columns, and
+// all warps combine the levels and store the layer's FP64 result.  The three phases follow one another:
+// the tile fills the shared memory (112 KB of A digits beside 56 KB of weights), and with the
+// FP64 pipe bound producer at 70-90 % of the time there is little to overlap.
+template <int D, int C, int KIND>
+__global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
+  constexpr int CR = JT<D>::CR;
+  constexpr int IPT = 128 / C;               // items per tile
+  constexpr bool kFwd = KIND <= LAY_FWD;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* As =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  unsigned char* Ws = As + kLayA;
+  __shared__ uint64_t done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int eA[128], eW[kLayW];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int ks_n = (p.K + 31) >> 5;
+  for (int idx = t; idx < kLayS * kLayW * 8; idx += kLayThreads) {   // 16-byte chunks
+    const int s = idx / (kLayW * 8), row = (idx >> 3) % kLayW, c8 = idx & 7;
+    *reinterpret_cast<uint4*>(Ws + s * kLayWSlice + swz(row, c8 * 8, kLayW)) =
+        *reinterpret_cast<const uint4*>(p.wsl + (size_t)idx * 16);
+  }
+  if (t < kLayW) eW[t] = p.we[t];
+  if (t == 0) {
+    mbar_init(&done, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "n"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  const int64_t tiles = (p.items + IPT - 1) / IPT;
+  uint32_t phase = 0;
+  bool ok = true;
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int64_t i0 = tile * IPT;
+    const int ni = (int)(p.items - i0 < IPT ? p.items - i0 : IPT);
+    // ---- A operand ---------------------------------------------------------------------------------
+    for (int it = warp; it < ni; it += kLayThreads / 32) {
+      const int64_t item = i0 + it;
+      const int64_t pt = kFwd ? item : item / p.nr;
+      double x[2][C];
+      unsigned m[C];
+#pragma unroll
+      for (int c = 0; c < C; c++) m[c] = 0;
+      double q = 0.0, beta = 0.0;
+      if (KIND == LAY_FWD_FIRST) {
+        q = p.qb[2 * pt];
+        beta = p.qb[2 * pt + 1];
+      }
+#pragma unroll
+      for (int s = 0; s < 2; s++) {
+        const int k = lane + 32 * s;
+#pragma unroll
+        for (int c = 0; c < C; c++) x[s][c] = 0.0;
+        if (k >= p.K) continue;
+        if constexpr (kFwd) {
+          double z[C];
+          if (KIND == LAY_FWD_FIRST) {
+            first_layer<D, C>(p.W0, p.b0, k, q, beta, z);
+          } else {
+#pragma unroll
+            for (int c = 0; c < C; c++) z[c] = p.zin[(pt * C + c) * p.K + k];
+            z[0] += p.bias[k];
+          }
+          tanh_jet<D, C>(z, x[s]);
+          if (p.hout) {
+#pragma unroll
+            for (int c = 0; c < CR; c++) p.hout[(pt * CR + c) * p.K + k] = x[s][c];
+          }
+        } else {
+          if (KIND == LAY_REV_LAST) {
+            for (int f = 0; f < p.nf; f++) {
+              const double w = p.Wlast[f * p.K + k];
+#pragma unroll
+              for (int c = 0; c < C; c++) x[s][c] = fma(w, p.seeds[(item * p.nf + f) * CR + c], x[s][c]);
+            }
+          } else {
+#pragma unroll
+            for (int c = 0; c < C; c++) x[s][c] = p.hbar[(item * C + c) * p.K + k];
+          }
+          double z[CR];
+#pragma unroll
+          for (int c = 1; c < CR; c++) z[c] = p.zin[(pt * p.cz + c) * p.K + k];
+          tanh_jet_adjoint<D>(p.hin[pt * CR * p.K + k], z, x[s]);
+#pragma unroll
+          for (int c = 0; c < C; c++) p.abar[(item * C + c) * p.K + k] = x[s][c];
+        }
+#pragma unroll
+        for (int c = 0; c < C; c++) {
+          const unsigned h = abs_hi(x[s][c]);
+          m[c] = h > m[c] ? h : m[c];
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < C; c++) {
+        const int row = it * C + c;
+        const int e = row_exponent(__reduce_max_sync(0xffffffffu, m[c]));
+        if (lane == 0) eA[row] = e;
+#pragma unroll
+        for (int s = 0; s < 2; s++) {
+          if (s < ks_n) {
+            const long long u = biased_digits(x[s][c], e == kLayBad ? 0 : e);
+            unsigned char* dst = As + swz(row, lane + 32 * s, 128);
+#pragma unroll
+            for (int d = 0; d < kLayS; d++)
+              *reinterpret_cast<unsigned short*>(dst + d * kLayASlice) = digit_bf16(u, d);
+          }
+        }
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMA reads what the threads wrote
+    tc_fence_before();
+    __syncthreads();
+    // ---- products ----------------------------------------------------------------------------------
+    if (t == 0) {
+      tc_fence_after();
+      const uint32_t a0 = smem_u32(As), w0 = smem_u32(Ws);
+#pragma unroll 1
+      for (int slot = 0; slot < kLayS; slot++)
+#pragma unroll 1
+        for (int s = 0; s <= slot; s++)
+          for (int ks = 0; ks < ks_n; ks++)
+#pragma unroll
+            for (int kk = 0; kk < 2; kk++)
+              mma_bf16<kLayW>(tmem + slot * kLayW, smem_desc(a0 + s * kLayASlice + ks * 128 * 64 + kk * 32),
+                              smem_desc(w0 + (slot - s) * kLayWSlice + ks * kLayW * 64 + kk * 32),
+                              (s == 0 && ks == 0 && kk == 0) ? 0u : 1u);
+      mma_commit(&done);
+    }
+    ok = __syncthreads_and(mbar_wait(&done, phase, p.flag, p.wait_ns));
+    phase ^= 1;
+    if (!ok) {   // the host sees the status bit; this CTA's remaining rows become NaN
+      for (; tile < tiles; tile += gridDim.x)
+        for (int64_t i = tile * IPT * C * p.N + t; i < (tile + 1) * IPT * C * p.N && i < p.items * C * p.N;
+             i += kLayThreads)
+          p.out[i] = nan("");
+      break;
+    }
+    tc_fence_after();
+    // ---- levels to FP64 ------------------------------------------------------------------------------
+    {
+      const int row = (warp & 3) * 32 + lane, cg = warp >> 2;   // 16 columns per warp
+      const bool valid = row < ni * C;
+      const int ea = eA[row];
+      const int64_t orow = i0 * C + row;
+#pragma unroll
+      for (int part = 0; part < 2; part++) {
+        const int col0 = cg * 16 + part * 8;
+        if (col0 >= p.N) continue;   // the same for the whole warp
+        uint32_t r[kLayS][8];
+#pragma unroll
+        for (int s = 0; s < kLayS; s++)
+          asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                       : "=r"(r[s][0]), "=r"(r[s][1]), "=r"(r[s][2]), "=r"(r[s][3]), "=r"(r[s][4]), "=r"(r[s][5]),
+                         "=r"(r[s][6]), "=r"(r[s][7])
+                       : "r"(tmem + ((uint32_t)((warp & 3) * 32) << 16) + s * kLayW + col0));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+          const int col = col0 + j;
+          int v[kLayS];
+#pragma unroll
+          for (int s = 0; s < kLayS; s++) v[s] = __float2int_rn(__uint_as_float(r[s][j]));
+          // sum_s v_s 256^(5 - s), the last level rounded in: |.| < 2^61
+          const long long hi = (long long)v[0] * 65536 + (v[1] * 256 + v[2]);
+          const long long lo = (long long)v[3] * 65536 + (v[4] * 256 + v[5]);
+          const long long T = (hi << 24) + lo + ((v[6] + 128) >> 8);
+          const int ew = eW[col];
+          const double d = (ea == kLayBad || ew == kLayBad) ? nan("") : scaled_int(T, ea + ew - 54);
+          if (valid && col < p.N) p.out[orow * p.N + col] = d;
+        }
+      }
+    }
+    tc_fence_before();   // the next tile's MMAs overwrite the accumulators after its barrier
+  }
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(512));
+  }
+}
+
+// ---- last hidden layer and the outputs --------------------------------------------------------------
+// One warp per point; the NF * C sums over the width are reduced by halving: after step o every
+// lane holds half as many partial sums, so NF * C sums cost about that many additions, not five
+// times as many.
+template <int D, int C, int NF>
+__global__ void __launch_bounds__(256) lay_last(int64_t npt, int K, const double* __restrict__ zin,
+                                                const double* __restrict__ bias, double* hout,
+                                                const double* __restrict__ W, const double* __restrict__ b,
+                                                double* nn) {
+  constexpr int CR = JT<D>::CR, V = NF * C;
+  constexpr int VP = V <= 2 ? 2 : V <= 4 ? 4 : V <= 8 ? 8 : V <= 16 ? 16 : 32;
+  const int lane = threadIdx.x & 31;
+  const int64_t pt = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (pt >= npt) return;
+  double v[VP];
+#pragma unroll
+  for (int i = 0; i < VP; i++) v[i] = 0.0;
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    const int k = lane + 32 * s;
+    if (k >= K) continue;
+    double z[C], h[C];
+#pragma unroll
+    for (int c = 0; c < C; c++) z[c] = zin[(pt * C + c) * K + k];
+    z[0] += bias[k];
+    tanh_jet<D, C>(z, h);
+    if (hout) {
+#pragma unroll
+      for (int c = 0; c < CR; c++) hout[(pt * CR + c) * K + k] = h[c];
+    }
+#pragma unroll
+    for (int f = 0; f < NF; f++) {
+      const double w = W[f * K + k];
+#pragma unroll
+      for (int c = 0; c < C; c++) v[f * C + c] = fma(w, h[c], v[f * C + c]);
+    }
+  }
+  int o = 16, idx = 0;
+#pragma unroll
+  for (int n = VP; n > 1; n >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < n / 2; i++) {
+      const double send = up ? v[i] : v[i + n / 2], keep = up ? v[i + n / 2] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    if (up) idx += n / 2;
+    o >>= 1;
+  }
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  constexpr int kDup = 32 / VP;   // lanes that hold the same sum
+  if (idx < V && lane % kDup == 0) nn[pt * V + idx] = v[0] + (idx % C == 0 ? b[idx / C] : 0.0);
+}
+
+// ---- residual chain ------------------------------------------------------------------------------------
+// One thread per (point, tangent direction): 32 points per warp, the directions over the block's
+// warps (direction 0: lambda; 1 + f C_R + c: output f, component c).  jet.cu evaluates the same
+// chain once per warp and point, its lanes being the directions, 19 of 32 at most.
+struct LayChain {
+  int64_t npt, p0;          // points of this chunk, the first one's index
+  const double* nn;         // [point][NF * CF]
+  double* seeds;            // [point][rows][NF * CR]
+  double* lamg;             // gradient mode: d / d lambda per point
+};
+template <int EQ, int MODE>
+__global__ void __launch_bounds__(MODE == MODE_RESIDUAL ? 128 : 32 * (1 + Eq<EQ>::NF * JT<Eq<EQ>::D>::CR))
+    lay_chain(const JetArgs A, const LayChain L) {
+  constexpr int D = Eq<EQ>::D, NF = Eq<EQ>::NF, NE = Eq<EQ>::NE, CR = JT<D>::CR;
+  constexpr int CF = (MODE == MODE_RESIDUAL) ? CR : JT<D>::CF;
+  const int dir = MODE == MODE_RESIDUAL ? 0 : threadIdx.y;
+  const int64_t pl = (MODE == MODE_RESIDUAL ? (int64_t)blockIdx.x * blockDim.y + threadIdx.y : blockIdx.x) * 32 +
+                     threadIdx.x;
+  if (pl >= L.npt) return;
+  const int64_t pt = L.p0 + pl;
+  const double lam = A.lamp ? *A.lamp : A.lam;
+  double y[D];
+  double u = 1.0;
+#pragma unroll
+  for (int k = 0; k < D; k++) y[k] = A.y[(int64_t)k * A.ystride + pt];
+#pragma unroll
+  for (int k = 0; k < D; k++) u = fma(y[k], y[k], u);
+  const bool tl = dir == 0 && MODE != MODE_RESIDUAL;
+  const Dl a = {1.0 / (1.0 + lam), tl ? -1.0 / ((1.0 + lam) * (1.0 + lam)) : 0.0};
+  const Dl q = pow_cb(u, -0.5 * a);
+  double beta = 0.0;
+  if (D == 2) beta = y[1] / sqrt(u);
+  const double* NN = L.nn + pl * (NF * CF);
+  Dl nn[NF][CR];
+#pragma unroll
+  for (int f = 0; f < NF; f++)
+#pragma unroll
+    for (int c = 0; c < CR; c++) {
+      double dv = 0.0;
+      if (MODE != MODE_RESIDUAL) {
+        if (dir == 0) dv = NN[f * CF + q_shift<D>(c)] * q.d;
+        else if (dir == 1 + f * CR + c) dv = 1.0;
+      }
+      nn[f][c] = {NN[f * CF + c], dv};
+    }
+  const Dl lamd = {lam, tl ? 1.0 : 0.0};
+  YJ<D> F[NF];
+  field_jets<EQ>(y, u, a, q, lamd, beta, nn, F);
+  Dl R[NE];
+  double sUv;
+  const int kind = A.kind;
+  residual_rows<EQ>(A, kind, pt, y, u, a, lamd, nn, F, R, sUv);
+  const int nrow = kind == KIND_INTERIOR ? NE : 1;
+  double w = A.wscale;
+  if (kind == KIND_INTERIOR && A.rho) w *= sqrt(A.rho[pt]);
+  const int64_t rbase = A.row0 + pt * nrow;
+  const bool su = EQ == GN_CCF && kind == KIND_INTERIOR && A.sU;
+  if (dir == 0) {
+#pragma unroll
+    for (int e = 0; e < NE; e++) {
+      if (e >= nrow) break;
+      const double rv = w * R[e].v;
+      if (A.r) A.r[rbase + e] = rv;
+      if (!isfinite(rv)) atomicOr(A.flag, 1);
+    }
+    if (su && MODE != MODE_GRADIENT) A.sU[pt] = w * sUv;
+  }
+  if (MODE == MODE_RESIDUAL) return;
+  if (MODE == MODE_JACOBIAN) {
+#pragma unroll
+    for (int e = 0; e < NE; e++) {
+      if (e >= nrow) break;
+      const double sd = w * R[e].d;
+      if (dir > 0) {
+        L.seeds[(pl * nrow + e) * (NF * CR) + dir - 1] = sd;
+      } else {
+        const int64_t row = rbase + e;
+        if (row >= A.jrow_lo && row < A.jrow_hi)
+          A.J[(row - A.jrow_lo) * A.ldJ + A.net.P] = A.lam_frozen ? 0.0 : sd;
+      }
+    }
+  } else {
+    double sd = 0.0;
+#pragma unroll
+    for (int e = 0; e < NE; e++) {
+      if (e >= nrow) break;
+      const double comb = A.seed ? A.seed[rbase + e] : w * R[e].v;
+      if (e == 0 && dir == 0 && su) A.sU[pt] = comb * w * sUv;
+      sd += comb * w * R[e].d;
+    }
+    if (dir > 0) L.seeds[pl * (NF * CR) + dir - 1] = sd;
+    else L.lamg[pl] = A.lam_frozen ? 0.0 : sd;
+  }
+}
+
+// ---- the first hidden layer's adjoint (no product follows it) -------------------------------------------
+template <int D>
+__global__ void __launch_bounds__(256) lay_first_adjoint(const LayArgs p) {
+  constexpr int CR = JT<D>::CR;
+  const int64_t n = p.items * p.K;
+  for (int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * 256) {
+    const int64_t item = idx / p.K;
+    const int k = (int)(idx - item * p.K);
+    double g[CR], z[CR];
+#pragma unroll
+    for (int c = 0; c < CR; c++) {
+      g[c] = p.hbar[(item * CR + c) * p.K + k];
+      z[c] = 0.0;
+    }
+    z[1] = p.W0[k * D];
+    if constexpr (D == 2) z[2] = p.W0[k * D + 1];
+    tanh_jet_adjoint<D>(p.hin[(item / p.nr) * CR * p.K + k], z, g);
+#pragma unroll
+    for (int c = 0; c < CR; c++) p.abar[(item * CR + c) * p.K + k] = g[c];
+  }
+}
+
+// ---- Jacobian rows -------------------------------------------------------------------------------------
+struct LayEntries {
+  NetDesc net;
+  int64_t npt, p0, row0, ldJ, jlo, jhi;
+  int nr;
+  const double* qb;
+  const double* H[GN_MAX_LAYERS + 1];      // [point][CR][w_j], j = 1 .. L - 1
+  const double* Ab[GN_MAX_LAYERS + 1];     // [item][CR][w_j]
+  const double* seeds;                     // [item][NF][CR]
+  double* J;
+};
+// One warp per (point, layer): the layer's activation jets stay in registers (two neurons per
+// lane) for all rows of the point, the adjoints are read at one address per warp, consecutive lanes
+// store consecutive columns.  FP64-bound: C_R multiply-adds per entry.
+template <int D>
+__global__ void __launch_bounds__(256) lay_entries(const LayEntries p) {
+  constexpr int CR = JT<D>::CR;
+  const int L = p.net.L, lane = threadIdx.x & 31;
+  const int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int64_t pl = w / L;
+  const int l = (int)(w - pl * L);
+  if (pl >= p.npt) return;
+  const int in = p.net.w[l], out = p.net.w[l + 1];
+  double h[2][CR];
+#pragma unroll
+  for (int s = 0; s < 2; s++)
+#pragma unroll
+    for (int c = 0; c < CR; c++) {
+      const int k = lane + 32 * s;
+      h[s][c] = (l > 0 && k < in) ? p.H[l][(pl * CR + c) * in + k] : 0.0;
+    }
+  for (int e = 0; e < p.nr; e++) {
+    const int64_t row = p.row0 + (p.p0 + pl) * p.nr + e;
+    if (row < p.jlo || row >= p.jhi) continue;
+    double* Jw = p.J + (row - p.jlo) * p.ldJ + p.net.offW[l];
+    double* Jb = p.J + (row - p.jlo) * p.ldJ + p.net.offB[l];
+    const int64_t item = pl * p.nr + e;
+    // adjoint component c of output o: ab[c * cs + o * os]
+    const double* ab = l < L - 1 ? p.Ab[l + 1] + item * CR * out : p.seeds + item * out * CR;
+    const int cs = l < L - 1 ? out : 1, os = l < L - 1 ? 1 : CR;
+    if (l == 0) {
+      const double q = p.qb[2 * pl], beta = p.qb[2 * pl + 1];
+      for (int o = lane; o < out; o += 32) {
+        const double a0 = ab[o];
+        Jw[o * D] = fma(a0, q, ab[out + o]);
+        if constexpr (D == 2) Jw[o * D + 1] = fma(a0, beta, ab[2 * out + o]);
+      }
+    } else {
+#pragma unroll 4
+      for (int o = 0; o < out; o++) {
+        double v0 = 0.0, v1 = 0.0;
+#pragma unroll
+        for (int c = 0; c < CR; c++) {
+          const double a = __ldg(ab + c * cs + o * os);
+          v0 = fma(a, h[0][c], v0);
+          if (in > 32) v1 = fma(a, h[1][c], v1);
+        }
+        if (lane < in) Jw[(int64_t)o * in + lane] = v0;
+        if (lane + 32 < in) Jw[(int64_t)o * in + lane + 32] = v1;
+      }
+    }
+    for (int o = lane; o < out; o += 32) Jb[o] = ab[o * os];
+  }
+}
+
+// ---- host side -----------------------------------------------------------------------------------------
+// Scratch of one point, in doubles.
+int64_t lay_point_doubles(const NetDesc& net, int d, int nf, int ne, int mode) {
+  const int cr = d == 1 ? 2 : 6, cf = mode == MODE_RESIDUAL ? cr : (d == 1 ? 3 : 9);
+  const int nr = mode == MODE_JACOBIAN ? ne : 1;
+  int64_t n = 2 + nf * cf;
+  for (int j = 1; j < net.L; j++) {
+    if (j >= 2) n += (int64_t)cf * net.w[j];
+    if (mode != MODE_RESIDUAL) n += (int64_t)cr * net.w[j] * (1 + nr);
+  }
+  if (mode != MODE_RESIDUAL) n += nr * nf * cr + 1 + 2 * (int64_t)nr * cr * kLayW;
+  return n;
+}
+constexpr int64_t kLayFixed = 2 * GN_MAX_LAYERS * (kLayS * kLayW * kLayW * 2 + kLayW * 4) + 8192;   // weight slices
+
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    const bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+                    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0;
+    return ok ? v : 152;
+  }();
+  return n;
+}
+
+template <int D, int C, int KIND>
+cudaError_t run_gemm(const LayArgs& a, cudaStream_t st) {
+  cudaError_t e =
+      cudaFuncSetAttribute(lay_gemm<D, C, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLaySmem);
+  if (e != cudaSuccess) return e;
+  const int64_t tiles = (a.items + 128 / C - 1) / (128 / C);
+  const int64_t grid = tiles < sm_count() ? tiles : sm_count();
+  lay_gemm<D, C, KIND><<<(unsigned)grid, kLayThreads, kLaySmem, st>>>(a);
+  count_launch();
+  return cudaGetLastError();
+}
+
+template <int EQ, int MODE>
+cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t st) {
+  constexpr int D = Eq<EQ>::D, NF = Eq<EQ>::NF, NE = Eq<EQ>::NE, CR = JT<D>::CR;
+  constexpr int C = (MODE == MODE_RESIDUAL) ? CR : JT<D>::CF;
+  const NetDesc& net = A.net;
+  const int L = net.L;
+  const int ne = A.kind == KIND_INTERIOR ? NE : 1;
+  const int nr = MODE == MODE_JACOBIAN ? ne : 1;
+  unsigned char* wsl = static_cast<unsigned char*>(ws);
+  int* we = reinterpret_cast<int*>(wsl + (size_t)2 * (L - 2) * kLayS * kLayW * kLayW * 2);
+  double* buf = reinterpret_cast<double*>(wsl + kLayFixed);
+  int64_t chunk = (int64_t)((ws_bytes - kLayFixed) / 8) / lay_point_doubles(net, D, NF, NE, MODE);
+  const int64_t wave = (int64_t)sm_count() * (128 / C);   // points of one round of forward tiles
+  if (chunk > 2 * wave) chunk = chunk / wave * wave;
+  const size_t opb = (size_t)kLayS * kLayW * kLayW * 2;
+  for (int64_t p0 = A.pt0; p0 < A.pt1; p0 += chunk) {
+    const int64_t n = p0 + chunk < A.pt1 ? chunk : A.pt1 - p0;
+    double* at = buf;
+    auto take = [&](int64_t per) {
+      double* r = at;
+      at += per * n;
+      return r;
+    };
+    double *Z[GN_MAX_LAYERS + 1] = {}, *H[GN_MAX_LAYERS + 1] = {}, *Ab[GN_MAX_LAYERS + 1] = {}, *hb[2] = {};
+    double* qb = take(2);
+    double* nn = take(NF * C);
+    for (int j = 2; j < L; j++) Z[j] = take((int64_t)C * net.w[j]);
+    double *seeds = nullptr, *lamg = nullptr;
+    if (MODE != MODE_RESIDUAL) {
+      for (int j = 1; j < L; j++) {
+        H[j] = take((int64_t)CR * net.w[j]);
+        Ab[j] = take((int64_t)nr * CR * net.w[j]);
+      }
+      seeds = take(nr * NF * CR);
+      lamg = take(1);
+      hb[0] = take((int64_t)nr * CR * kLayW);
+      hb[1] = take((int64_t)nr * CR * kLayW);
+    }
+    LayPrep pr;
+    pr.y = A.y;
+    pr.ystride = A.ystride;
+    pr.pt0 = p0;
+    pr.npt = n;
+    pr.lam = A.lam;
+    pr.lamp = A.lamp;
+    pr.qb = qb;
+    pr.theta = A.theta;
+    pr.net = net;
+    pr.wsl = wsl;
+    pr.we = we;
+    pr.pt_blocks = (int)((n + 255) / 256);
+    const int wblocks = p0 == A.pt0 ? (L - 2) * 2 * kLayW / 8 : 0;   // the weights once per pass
+    lay_inputs<D><<<pr.pt_blocks + wblocks, 256, 0, st>>>(pr);
+    count_launch();
+    LayArgs g;
+    memset(&g, 0, sizeof(g));
+    g.nf = NF;
+    g.cz = C;
+    g.nr = nr;
+    g.qb = qb;
+    g.W0 = A.theta + net.offW[0];
+    g.b0 = A.theta + net.offB[0];
+    g.Wlast = A.theta + net.offW[L - 1];
+    g.flag = A.flag + 2;
+    g.wait_ns = g_oz_wait_ns.load(std::memory_order_relaxed);
+    cudaError_t e = cudaSuccess;
+    for (int j = 1; j <= L - 2 && e == cudaSuccess; j++) {
+      g.items = n;
+      g.K = net.w[j];
+      g.N = net.w[j + 1];
+      g.zin = Z[j];
+      g.bias = A.theta + net.offB[j - 1];
+      g.hout = H[j];
+      g.out = Z[j + 1];
+      g.wsl = wsl + (size_t)(2 * (j - 1)) * opb;
+      g.we = we + 2 * (j - 1) * kLayW;
+      e = j == 1 ? run_gemm<D, C, LAY_FWD_FIRST>(g, st) : run_gemm<D, C, LAY_FWD>(g, st);
+    }
+    if (e != cudaSuccess) return e;
+    lay_last<D, C, NF><<<(unsigned)((n + 7) / 8), 256, 0, st>>>(n, net.w[L - 1], Z[L - 1],
+                                                                A.theta + net.offB[L - 2], H[L - 1],
+                                                                A.theta + net.offW[L - 1],
+                                                                A.theta + net.offB[L - 1], nn);
+    count_launch();
+    LayChain ch = {n, p0, nn, seeds, lamg};
+    const dim3 cb(32, MODE == MODE_RESIDUAL ? 4 : 1 + NF * CR);
+    const int64_t cpts = MODE == MODE_RESIDUAL ? 128 : 32;
+    lay_chain<EQ, MODE><<<(unsigned)((n + cpts - 1) / cpts), cb, 0, st>>>(A, ch);
+    count_launch();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (MODE == MODE_RESIDUAL) continue;
+    const double* hbar = nullptr;
+    for (int j = L - 2; j >= 1; j--) {
+      g.items = n * nr;
+      g.K = net.w[j + 1];
+      g.N = net.w[j];
+      g.zin = Z[j + 1];
+      g.hin = H[j + 1];
+      g.seeds = seeds;
+      g.hbar = hbar;
+      g.abar = Ab[j + 1];
+      g.out = hb[j & 1];
+      g.wsl = wsl + (size_t)(2 * (j - 1) + 1) * opb;
+      g.we = we + (2 * (j - 1) + 1) * kLayW;
+      e = j == L - 2 ? run_gemm<D, CR, LAY_REV_LAST>(g, st) : run_gemm<D, CR, LAY_REV>(g, st);
+      if (e != cudaSuccess) return e;
+      hbar = hb[j & 1];
+    }
+    g.K = net.w[1];
+    g.hin = H[1];
+    g.hbar = hbar;
+    g.abar = Ab[1];
+    {
+      int64_t blocks = (g.items * g.K + 255) / 256;
+      if (blocks > 16 * sm_count()) blocks = 16 * sm_count();
+      lay_first_adjoint<D><<<(unsigned)blocks, 256, 0, st>>>(g);
+      count_launch();
+    }
+    LayEntries en;
+    memset(&en, 0, sizeof(en));
+    en.net = net;
+    en.npt = n;
+    en.p0 = p0;
+    en.row0 = A.row0;
+    en.ldJ = A.ldJ;
+    en.jlo = A.jrow_lo;
+    en.jhi = A.jrow_hi;
+    en.nr = nr;
+    en.qb = qb;
+    for (int j = 1; j < L; j++) {
+      en.H[j] = H[j];
+      en.Ab[j] = Ab[j];
+    }
+    en.seeds = seeds;
+    en.J = A.J;
+    lay_entries<D><<<(unsigned)((n * L + 7) / 8), 256, 0, st>>>(en);
+    count_launch();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+template <int EQ>
+cudaError_t layers_mode(const JetArgs& a, void* ws, size_t bytes, cudaStream_t st) {
+  return a.mode == MODE_RESIDUAL ? layers_eq<EQ, MODE_RESIDUAL>(a, ws, bytes, st)
+                                 : layers_eq<EQ, MODE_JACOBIAN>(a, ws, bytes, st);
+}
+
+}  // namespace
+
+// The layered path takes tanh networks of at least two hidden layers, none wider than the 64
+// columns of its tiles or narrower than 24, and point sets (all of them, not a row block's, so that
+// a block's rows equal the whole's) of 2048 points in 2D, 4096 in 1D.  Below that its chain of
+// 2 L launches takes longer than one pointwise kernel.  Pointwise / layered time, residual and
+// Jacobian pass: 1D width 32 x 2, 2048 points 44 / 54 and 79 / 111 us, 4096 points 79 / 58 and 147 / 133;
+// 1D 64 x 3, 8192 points 390 / 128 and 1120 / 541; 2D IPM 32 x 2, 1024 points 54 / 58 and 142 / 196, 2048 points
+// 106 / 62 and 304 / 282; IPM 64 x 3, 8192 points 1170 / 260 and 5119 / 2619.  Width 16 x 3, IPM, 8192 points:
+// 332 / 181 and 911 / 1063 (the products are padded to 64 columns).
+static bool layers_net(const NetDesc& net) {
+  if (net.fourier || net.exp_out || net.L < 3) return false;
+  for (int l = 1; l < net.L; l++)
+    if (net.w[l] > kLayW || net.w[l] < 24) return false;
+  return true;
+}
+static int64_t layers_min_points(int d) { return d == 1 ? 4096 : 2048; }
+
+bool layers_eligible(const JetArgs& a) {
+  if (a.mode == MODE_GRADIENT || a.kind == KIND_PROBE) return false;
+  return a.n >= layers_min_points(a.net.w[0]) && layers_net(a.net);
+}
+
+size_t layers_ws_bytes(const NetDesc& net, int d, int nf, int ne, int64_t npt) {
+  if (npt < layers_min_points(d) || !layers_net(net)) return 0;
+  const int64_t per = lay_point_doubles(net, d, nf, ne, MODE_JACOBIAN) * 8;
+  const int64_t cap = (int64_t)320 << 20;
+  return (size_t)(kLayFixed + (per * npt < cap ? per * npt : cap));
+}
+
+cudaError_t launch_layers(const JetArgs& a, void* ws, size_t ws_bytes, cudaStream_t st) {
+  if (a.pt1 <= a.pt0) return cudaSuccess;
+  switch (a.eq) {
+    case GN_BURGERS: return layers_mode<GN_BURGERS>(a, ws, ws_bytes, st);
+    case GN_CCF: return layers_mode<GN_CCF>(a, ws, ws_bytes, st);
+    case GN_IPM: return layers_mode<GN_IPM>(a, ws, ws_bytes, st);
+    case GN_BOUSSINESQ: return layers_mode<GN_BOUSSINESQ>(a, ws, ws_bytes, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace gn

@@ -1,0 +1,114 @@
+"""The layered passes (many points, hidden layers as split products on the tensor cores) against the
+one-warp-per-point kernel, which takes the same points when there are few of them.
+
+A row depends on its own point (and, for CCF, on the Hilbert nodes, the same in both problems), so
+the rows of a large problem at some of its points equal those of a problem of these points alone,
+up to the factor sqrt(N_small / N_large) of the row weights."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2509_14185_gb300 import inputs as I
+from tests.gpu_cases import TOL, col_rel, dev, gpu_problem, host, rel
+
+pytestmark = [pytest.mark.gpu, pytest.mark.filterwarnings("ignore::RuntimeWarning")]
+
+EQS = {"burgers": (I.BURGERS, 1), "ccf": (I.CCF, 1), "ipm": (I.IPM, 2), "boussinesq": (I.BOUSSINESQ, 3)}
+
+
+def _pair(name, hidden, n, n_bnd=40, seed=3, **kw):
+    eq, nf = EQS[name]
+    big = I.weighted(I.small_case(eq, [I.EQUATION_DIM[eq]] + hidden + [nf], n, n_bnd=n_bnd if nf > 1 else 0, seed=seed))
+    pick = np.unique(np.concatenate([[0, 1, n // 2, n - 2, n - 1], np.arange(0, n, 37)]))
+    few = dataclasses.replace(big, y=np.ascontiguousarray(big.y[:, pick]), rho=big.rho[pick])
+    return big, few, pick, gpu_problem(big, **kw), gpu_problem(few, **kw)
+
+
+def _rows(pick, ne):
+    return (pick[:, None] * ne + np.arange(ne)).reshape(-1)
+
+
+# tiles of 128 rows hold 64, 42, 21 or 14 items; widths with one or two 32-wide stages, ragged ones
+@pytest.mark.parametrize("name,hidden,n", [
+    ("burgers", [24, 24], 4096), ("burgers", [32, 64, 33], 4111), ("ccf", [64, 64, 64], 4097), ("ccf", [31, 25], 4099),
+    ("ipm", [64, 64, 64, 64], 2049), ("ipm", [40, 27, 64], 2200), ("boussinesq", [48, 48, 48], 2048),
+    ("boussinesq", [33, 64], 2061)])
+def test_rows_and_jacobian_equal_the_pointwise_kernel(name, hidden, n):
+    big, few, pick, pb, pf = _pair(name, hidden, n)
+    ne = EQS[name][1]
+    sel = torch.from_numpy(_rows(pick, ne)).cuda()
+    scale = np.sqrt(len(pick) / n)
+    th = dev(big.theta)
+    m = len(pick) * ne
+    r_b, r_f = pb.residual(th, big.lam)[0], pf.residual(th, big.lam)[0]
+    assert rel(host(r_b[sel]), scale * host(r_f[:m])) <= TOL
+    J_b = pb.jacobian(th, big.lam)
+    J_f = scale * host(pf.jacobian(th, big.lam)[:m])
+    J_s = host(J_b[sel])
+    assert rel(J_s, J_f) <= TOL
+    assert col_rel(J_s, J_f, floor=1e-300) <= TOL
+    # a block that starts and ends inside a point equals the same rows of the whole
+    lo, cnt = n // 3 * ne + 1, n // 2 * ne
+    assert torch.equal(pb.jacobian(th, big.lam, row0=lo, nrows=cnt, ld=pb.P + 9), J_b[lo:lo + cnt])
+
+
+def test_many_wall_points_equal_few():
+    """2050 wall points take the layered path, 900 of them the pointwise one."""
+    big, _, _, pb, _ = _pair("ipm", [32, 32, 32], 300, n_bnd=2050)
+    pf = gpu_problem(dataclasses.replace(big, y_bnd=np.ascontiguousarray(big.y_bnd[:, :900])))
+    th = dev(big.theta)
+    s = np.sqrt(900 / 2050)
+    r_b, r_f = pb.residual(th, big.lam)[0], pf.residual(th, big.lam)[0]
+    assert torch.equal(r_b[:600], r_f[:600]) and torch.equal(r_b[-1:], r_f[-1:])
+    assert rel(host(r_b[600:1500]), s * host(r_f[600:1500])) <= TOL
+    J_b, J_f = host(pb.jacobian(th, big.lam, 600, 900)), s * host(pf.jacobian(th, big.lam, 600, 900))
+    assert rel(J_b, J_f) <= TOL
+
+
+@pytest.mark.parametrize("name,hidden", [("burgers", [24, 24]), ("ipm", [30, 30, 30])])
+def test_second_stage(name, hidden):
+    n = 4100 if name == "burgers" else 2300
+    big, few, pick, pb, pf = _pair(name, hidden, n)
+    ne = EQS[name][1]
+    w1 = [I.EQUATION_DIM[big.equation], 9, EQS[name][1]]
+    for p in (pb, pf):
+        p.gn_set_stage1(w1, dev(I.xavier_init(w1, 5)), big.lam, 1e-3)
+    th = dev(big.theta)
+    sel = torch.from_numpy(_rows(pick, ne)).cuda()
+    J_s, J_f = host(pb.jacobian(th, big.lam)[sel]), host(pf.jacobian(th, big.lam)[:len(pick) * ne])
+    assert rel(J_s, np.sqrt(len(pick) / n) * J_f) <= TOL
+
+
+@pytest.mark.parametrize("name", ["burgers", "boussinesq"])
+def test_extreme_and_non_finite_values(name):
+    """Saturated and tiny weights reach the digits' limits; a NaN weight or point reaches its rows."""
+    big, few, pick, pb, pf = _pair(name, [40, 40, 40], 4200)
+    ne = EQS[name][1]
+    sel = torch.from_numpy(_rows(pick, ne)).cuda()
+    theta = big.theta.copy()
+    theta[::7] *= 40.0
+    theta[3::11] *= 1e-200
+    th = dev(theta)
+    m = len(pick) * ne
+    r_s, r_f = host(pb.residual(th, big.lam)[0][sel]), host(pf.residual(th, big.lam)[0][:m])
+    assert np.all(np.isfinite(r_f))
+    assert rel(r_s, np.sqrt(len(pick) / 4200) * r_f) <= TOL
+    theta[300] = np.nan
+    assert pb.gn_residual(dev(theta), big.lam)[0] == -4
+    y = big.y.copy()
+    y[0, 1234] = np.nan
+    pn = gpu_problem(dataclasses.replace(big, y=y))
+    r = pn.new_vec(pn.n_rows)
+    assert pn.gn_residual(dev(big.theta), big.lam, r)[0] == -4
+    bad = np.flatnonzero(~np.isfinite(host(r)))
+    assert bad.size and set(bad) <= set(range(1234 * ne, 1234 * ne + ne))
+
+
+def test_step_graph_equals_step():
+    big, _, _, pb, _ = _pair("ccf", [32, 32], 4300, precision=2, n_slices=6)
+    pg = gpu_problem(big, precision=2, n_slices=6)
+    ta, tb = dev(big.theta), dev(big.theta)
+    a, b = pb.gn_step(ta, big.lam, 1e-2), pg.gn_step_graph(tb, big.lam, 1e-2)
+    assert a[:3] == b[:3] and torch.equal(ta, tb)
