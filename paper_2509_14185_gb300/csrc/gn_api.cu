@@ -160,9 +160,19 @@ int run_pass(gn_handle* h, const double* theta, double lam, const Pass& ps, doub
 
   // wall points and the normalisation row: rows of their own.  In residual and Jacobian
   // modes they run on the handle's side stream, beside the Hilbert nodes and the interior
-  // (a one-point pass is latency-bound; alone it would add its whole latency); gradient mode
-  // accumulates every kind into the same per-warp partials, so it keeps them in order.
-  const bool side = ps.mode != MODE_GRADIENT && h->st_aux;
+  // (a one-point pass is latency-bound; alone it would add its whole latency); in gradient mode
+  // the pointwise kernel accumulates every kind into the same per-warp partials, so that they keep
+  // their order unless no other kind takes that kernel.
+  bool side = h->st_aux != nullptr;
+  if (ps.mode == MODE_GRADIENT) {
+    JetArgs b = a;
+    b.kind = KIND_INTERIOR;
+    b.n = n;
+    const bool layered = takes_layers(h, b);
+    side = side && layered && h->eq != GN_CCF && h->p.n_d1 == 0 && h->p.n_d2 == 0;
+    if (h->lay_ws)
+      GN_TRY_CUDA(cudaMemsetAsync(layers_parts(h->lay_ws), 0, layers_part_count() * a.ldg * 8, st));
+  }
   auto wall_rows = [&](cudaStream_t sx, bool layered) -> int {
     if (h->p.n_bnd > 0) {
       JetArgs b = a;
@@ -400,7 +410,8 @@ int run_pass(gn_handle* h, const double* theta, double lam, const Pass& ps, doub
       b.base_ld = 1;
       GN_TRY_CUDA(launch_jet(b, st, nullptr));
     }
-    GN_TRY_CUDA(launch_gpart_reduce(h->gpart, h->gpart_warps, a.ldg, h->Pp, grad, 0, st));
+    GN_TRY_CUDA(launch_gpart_reduce(h->gpart, h->gpart_warps, h->lay_ws ? layers_parts(h->lay_ws) : nullptr,
+                                    h->lay_ws ? layers_part_count() : 0, a.ldg, h->Pp, grad, st));
   }
   return GN_OK;
 }

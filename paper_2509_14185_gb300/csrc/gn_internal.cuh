@@ -230,6 +230,10 @@ cudaError_t launch_jet(const JetArgs& a, cudaStream_t st, int64_t* warps_used);
 bool layers_eligible(const JetArgs& a);
 size_t layers_ws_bytes(const NetDesc& net, int d, int nf, int ne, int64_t npt);
 cudaError_t launch_layers(const JetArgs& a, void* ws, size_t ws_bytes, cudaStream_t st);
+// gradient mode: the layered passes' partial gradients [layers_part_count][ldg] in ws (accumulated;
+// the caller clears them before the first launch)
+double* layers_parts(void* ws);
+int layers_part_count();
 // derivative-loss rows of order ord (1: d1, 2: d2) at the a.n points (djet.cu); a.row0 is the
 // first row, a.wscale sqrt(2 c_d / (N_d N_E d^ord)).  CCF: a.ug / a.dcoef hold the K part's
 // and D's Taylor coefficients in y ([m][n], m <= order_y), a.sU receives d row / d U_m ([m][n],
@@ -238,8 +242,9 @@ cudaError_t launch_djet(const JetArgs& a, int ord, cudaStream_t st, int64_t* war
 // degree in y of the field series of the derivative rows of order ord in d dimensions
 inline int djet_order_y(int d, int ord) { return (d == 1 ? 1 : 2) + ord; }
 int jet_gpart_warps(const NetDesc& net, int d, int nf, int64_t n_max);
-cudaError_t launch_gpart_reduce(const double* gpart, int64_t warps, int64_t ldg, int64_t n,
-                                double* out, int accumulate, cudaStream_t st);
+// out[0..n) = the sum of the rows of gpart and, with parts, of the rows of parts
+cudaError_t launch_gpart_reduce(const double* gpart, int64_t warps, const double* parts, int64_t nparts, int64_t ldg,
+                                int64_t n, double* out, cudaStream_t st);
 
 // FP64 GEMM: C(m x n) = alpha * sum_k A(m,k) B(k,n) + beta * C, optional row scale.
 // a_kcontig: A(m,k) = A[m*lda + k] (else A[k*lda + m]); b_kcontig: B(k,n) = B[n*ldb + k]

@@ -384,12 +384,26 @@ __global__ void transpose_weights_kernel(const NetDesc net, const double* __rest
   }
 }
 
-__global__ void gpart_reduce_kernel(const double* __restrict__ gpart, int64_t warps, int64_t ldg, int64_t n,
-                                    double* out, int accumulate) {
-  for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < n; a += (int64_t)gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int64_t w = 0; w < warps; w++) s += gpart[w * ldg + a];
-    out[a] = accumulate ? out[a] + s : s;
+// Column sums of the partial gradients, 32 columns per block: 32 warps take every 32nd row (coalesced),
+// their sums are added in warp order.  (One thread per column took 542 us for 2432 rows of 5000.)
+__global__ void __launch_bounds__(1024) gpart_reduce_kernel(const double* __restrict__ gpart, int64_t warps,
+                                                            const double* __restrict__ parts, int64_t nparts,
+                                                            int64_t ldg, int64_t n, double* out) {
+  __shared__ double s[32][33];
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int64_t a = (int64_t)blockIdx.x * 32 + lane;
+  double v = 0.0;
+  if (a < n) {
+    for (int64_t w = g; w < warps; w += 32) v += gpart[w * ldg + a];
+    for (int64_t w = g; w < nparts; w += 32) v += parts[w * ldg + a];
+  }
+  s[g][lane] = v;
+  __syncthreads();
+  if (g == 0 && a < n) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < 32; w++) t += s[w][lane];
+    out[a] = t;
   }
 }
 
@@ -486,12 +500,9 @@ cudaError_t launch_transpose_weights(const NetDesc& net, const double* theta, do
   return cudaGetLastError();
 }
 
-cudaError_t launch_gpart_reduce(const double* gpart, int64_t warps, int64_t ldg, int64_t n, double* out,
-                                int accumulate, cudaStream_t st) {
-  int64_t blocks = (n + 255) / 256;
-  if (blocks > 1024) blocks = 1024;
-  if (blocks < 1) blocks = 1;
-  gpart_reduce_kernel<<<(unsigned)blocks, 256, 0, st>>>(gpart, warps, ldg, n, out, accumulate);
+cudaError_t launch_gpart_reduce(const double* gpart, int64_t warps, const double* parts, int64_t nparts, int64_t ldg,
+                                int64_t n, double* out, cudaStream_t st) {
+  gpart_reduce_kernel<<<(unsigned)((n + 31) / 32), 1024, 0, st>>>(gpart, warps, parts, nparts, ldg, n, out);
   count_launch();
   return cudaGetLastError();
 }

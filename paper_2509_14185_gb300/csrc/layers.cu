@@ -14,7 +14,8 @@
 //                 reverse-pass seeds (chain.cuh, the chain jet.cu evaluates per warp)
 //   lay_gemm      reverse, per hidden layer: abar_{j+1} = Hbar_{j+1} through the tanh jets,
 //                 Hbar_j = W_j^T abar_{j+1}
-//   lay_entries   the Jacobian rows sum_c abar_c[o] h_c[i]
+//   lay_entries   the Jacobian rows sum_c abar_c[o] h_c[i]; or, for the gradient, their sums over the
+//                 points (lay_outer, lay_sums)
 //
 // Precision of the products: every row of either operand is scaled by a power of two and rounded to
 // a 55-bit integer (its largest element keeps two bits more than FP64's own 53), written as 7
@@ -678,6 +679,115 @@ __global__ void __launch_bounds__(256) lay_entries(const LayEntries p) {
   }
 }
 
+// ---- gradient ------------------------------------------------------------------------------------------
+// Adjoint mode sums the same products over the points: the weights of layer l get
+// sum_(point, c) abar_(l+1)[c][o] h_l[c][i], the rest are sums over the points alone.  The points are
+// cut into kLayParts parts, each with its own partial gradient (added in part order at the end).
+constexpr int kLayParts = 64;
+struct LayGrad {
+  LayEntries e;
+  const double* lamg;
+  double* parts;            // [kLayParts][ldg], accumulated
+  int64_t ldg;
+};
+// Hidden-to-hidden weights: one block per 16 x 16 outputs and part, eight groups of 64 threads
+// (2 x 2 outputs each) sharing the rows (point, c).  FP64-bound; 16-wide tiles pad the usual widths
+// (48, 64) not at all.
+template <int D>
+__global__ void __launch_bounds__(512) lay_outer(const LayGrad p) {
+  constexpr int CR = JT<D>::CR, KG = 8;
+  __shared__ double As[KG][16][17], Bs[KG][16][17];
+  int l = 1, tile = blockIdx.x;
+  for (; l < p.e.net.L - 1; l++) {
+    const int nt = ((p.e.net.w[l] + 15) / 16) * ((p.e.net.w[l + 1] + 15) / 16);
+    if (tile < nt) break;
+    tile -= nt;
+  }
+  const int in = p.e.net.w[l], out = p.e.net.w[l + 1], ti = (in + 15) / 16;
+  const int o0 = tile / ti * 16, i0 = tile % ti * 16;
+  const int64_t R = p.e.npt * CR, per = (R + kLayParts - 1) / kLayParts;
+  const int64_t r0 = blockIdx.y * per, r1 = r0 + per < R ? r0 + per : R;
+  const double* A = p.e.Ab[l + 1];
+  const double* B = p.e.H[l];
+  const int t = threadIdx.x & 63, kg = threadIdx.x >> 6, tx = t & 7, ty = t >> 3;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  for (int64_t k0 = r0; k0 < r1; k0 += KG * 16) {
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const int kk = (t >> 4) + 4 * q, cc = t & 15;
+      const int64_t r = k0 + kg * 16 + kk;
+      As[kg][kk][cc] = (r < r1 && o0 + cc < out) ? A[r * out + o0 + cc] : 0.0;
+      Bs[kg][kk][cc] = (r < r1 && i0 + cc < in) ? B[r * in + i0 + cc] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < 16; kk++) {
+      const double a0 = As[kg][kk][ty], a1 = As[kg][kk][ty + 8], b0 = Bs[kg][kk][tx], b1 = Bs[kg][kk][tx + 8];
+      acc[0][0] = fma(a0, b0, acc[0][0]);
+      acc[0][1] = fma(a0, b1, acc[0][1]);
+      acc[1][0] = fma(a1, b0, acc[1][0]);
+      acc[1][1] = fma(a1, b1, acc[1][1]);
+    }
+    __syncthreads();
+  }
+  // the groups' sums in group order
+  double* sum = &As[0][0][0];
+#pragma unroll
+  for (int q = 0; q < 4; q++) sum[(q * KG + kg) * 64 + t] = acc[q >> 1][q & 1];
+  __syncthreads();
+  if (threadIdx.x < 256) {
+    const int q = threadIdx.x >> 6;
+    double v = 0.0;
+#pragma unroll
+    for (int g = 0; g < KG; g++) v += sum[(q * KG + g) * 64 + t];
+    const int o = o0 + ty + 8 * (q >> 1), i = i0 + tx + 8 * (q & 1);
+    if (o < out && i < in) p.parts[blockIdx.y * p.ldg + p.e.net.offW[l] + (int64_t)o * in + i] += v;
+  }
+}
+// First and last layer's weights, the biases and lambda: one thread per entry and part.
+template <int D>
+__global__ void __launch_bounds__(256) lay_sums(const LayGrad p) {
+  constexpr int CR = JT<D>::CR;
+  const NetDesc& net = p.e.net;
+  const int L = net.L;
+  const int64_t per = (p.e.npt + kLayParts - 1) / kLayParts;
+  const int64_t p0 = blockIdx.y * per, p1 = p0 + per < p.e.npt ? p0 + per : p.e.npt;
+  int idx = blockIdx.x * 256 + threadIdx.x;
+  double v = 0.0;
+  int64_t at = -1;
+  if (idx < net.w[1] * D) {
+    const int o = idx / D, i = idx % D;
+    const double* a = p.e.Ab[1] + o;
+    for (int64_t q = p0; q < p1; q++)
+      v += fma(a[q * CR * net.w[1]], p.e.qb[2 * q + i], a[(q * CR + 1 + i) * net.w[1]]);
+    at = net.offW[0] + idx;
+  } else if ((idx -= net.w[1] * D) < net.w[L] * net.w[L - 1]) {
+    const int f = idx / net.w[L - 1], i = idx % net.w[L - 1];
+    for (int64_t q = p0; q < p1; q++)
+#pragma unroll
+      for (int c = 0; c < CR; c++)
+        v = fma(p.e.seeds[(q * net.w[L] + f) * CR + c], p.e.H[L - 1][(q * CR + c) * net.w[L - 1] + i], v);
+    at = net.offW[L - 1] + idx;
+  } else if ((idx -= net.w[L] * net.w[L - 1]) == 0) {
+    for (int64_t q = p0; q < p1; q++) v += p.lamg[q];
+    at = net.P;
+  } else {
+    idx -= 1;
+    for (int l = 0; l < L; l++) {
+      const int out = net.w[l + 1];
+      if (idx < out) {
+        const double* a = l < L - 1 ? p.e.Ab[l + 1] + idx : p.e.seeds + idx * CR;
+        const int64_t step = l < L - 1 ? CR * out : out * CR;
+        for (int64_t q = p0; q < p1; q++) v += a[q * step];
+        at = net.offB[l] + idx;
+        break;
+      }
+      idx -= out;
+    }
+  }
+  if (at >= 0) p.parts[blockIdx.y * p.ldg + at] += v;
+}
+
 // ---- host side -----------------------------------------------------------------------------------------
 // Scratch of one point, in doubles.
 int64_t lay_point_doubles(const NetDesc& net, int d, int nf, int ne, int mode) {
@@ -691,6 +801,8 @@ int64_t lay_point_doubles(const NetDesc& net, int d, int nf, int ne, int mode) {
   if (mode != MODE_RESIDUAL) n += nr * nf * cr + 1 + 2 * (int64_t)nr * cr * kLayW;
   return n;
 }
+int64_t lay_ldg(const NetDesc& net) { return (net.P + 1 + 15) / 16 * 16; }
+int64_t lay_parts_doubles(const NetDesc& net) { return kLayParts * lay_ldg(net); }
 constexpr int64_t kLayFixed = 2 * GN_MAX_LAYERS * (kLayS * kLayW * kLayW * 2 + kLayW * 4) + 8192;   // weight slices
 
 int sm_count() {
@@ -725,8 +837,10 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
   const int nr = MODE == MODE_JACOBIAN ? ne : 1;
   unsigned char* wsl = static_cast<unsigned char*>(ws);
   int* we = reinterpret_cast<int*>(wsl + (size_t)2 * (L - 2) * kLayS * kLayW * kLayW * 2);
-  double* buf = reinterpret_cast<double*>(wsl + kLayFixed);
-  int64_t chunk = (int64_t)((ws_bytes - kLayFixed) / 8) / lay_point_doubles(net, D, NF, NE, MODE);
+  double* parts = reinterpret_cast<double*>(wsl + kLayFixed);
+  double* buf = parts + lay_parts_doubles(net);
+  int64_t chunk = (int64_t)((ws_bytes - kLayFixed) / 8 - lay_parts_doubles(net)) /
+                  lay_point_doubles(net, D, NF, NE, MODE);
   const int64_t wave = (int64_t)sm_count() * (128 / C);   // points of one round of forward tiles
   if (chunk > 2 * wave) chunk = chunk / wave * wave;
   const size_t opb = (size_t)kLayS * kLayW * kLayW * 2;
@@ -850,6 +964,20 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
     }
     en.seeds = seeds;
     en.J = A.J;
+    if (MODE == MODE_GRADIENT) {
+      LayGrad gr = {en, lamg, parts, lay_ldg(net)};
+      int tiles = 0, sums = net.w[1] * D + net.w[L] * net.w[L - 1] + 1;
+      for (int l = 0; l < L; l++) {
+        if (l >= 1 && l < L - 1) tiles += ((net.w[l] + 15) / 16) * ((net.w[l + 1] + 15) / 16);
+        sums += net.w[l + 1];
+      }
+      lay_outer<D><<<dim3((unsigned)tiles, kLayParts), 512, 0, st>>>(gr);
+      count_launch();
+      lay_sums<D><<<dim3((unsigned)((sums + 255) / 256), kLayParts), 256, 0, st>>>(gr);
+      count_launch();
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      continue;
+    }
     lay_entries<D><<<(unsigned)((n * L + 7) / 8), 256, 0, st>>>(en);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -859,8 +987,11 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
 
 template <int EQ>
 cudaError_t layers_mode(const JetArgs& a, void* ws, size_t bytes, cudaStream_t st) {
-  return a.mode == MODE_RESIDUAL ? layers_eq<EQ, MODE_RESIDUAL>(a, ws, bytes, st)
-                                 : layers_eq<EQ, MODE_JACOBIAN>(a, ws, bytes, st);
+  switch (a.mode) {
+    case MODE_RESIDUAL: return layers_eq<EQ, MODE_RESIDUAL>(a, ws, bytes, st);
+    case MODE_JACOBIAN: return layers_eq<EQ, MODE_JACOBIAN>(a, ws, bytes, st);
+    default: return layers_eq<EQ, MODE_GRADIENT>(a, ws, bytes, st);
+  }
 }
 
 }  // namespace
@@ -882,16 +1013,17 @@ static bool layers_net(const NetDesc& net) {
 static int64_t layers_min_points(int d) { return d == 1 ? 4096 : 2048; }
 
 bool layers_eligible(const JetArgs& a) {
-  if (a.mode == MODE_GRADIENT || a.kind == KIND_PROBE) return false;
-  return a.n >= layers_min_points(a.net.w[0]) && layers_net(a.net);
+  return a.kind != KIND_PROBE && a.n >= layers_min_points(a.net.w[0]) && layers_net(a.net);
 }
 
 size_t layers_ws_bytes(const NetDesc& net, int d, int nf, int ne, int64_t npt) {
   if (npt < layers_min_points(d) || !layers_net(net)) return 0;
   const int64_t per = lay_point_doubles(net, d, nf, ne, MODE_JACOBIAN) * 8;
   const int64_t cap = (int64_t)320 << 20;
-  return (size_t)(kLayFixed + (per * npt < cap ? per * npt : cap));
+  return (size_t)(kLayFixed + lay_parts_doubles(net) * 8 + (per * npt < cap ? per * npt : cap));
 }
+double* layers_parts(void* ws) { return reinterpret_cast<double*>(static_cast<unsigned char*>(ws) + kLayFixed); }
+int layers_part_count() { return kLayParts; }
 
 cudaError_t launch_layers(const JetArgs& a, void* ws, size_t ws_bytes, cudaStream_t st) {
   if (a.pt1 <= a.pt0) return cudaSuccess;

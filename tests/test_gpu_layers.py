@@ -54,6 +54,27 @@ def test_rows_and_jacobian_equal_the_pointwise_kernel(name, hidden, n):
     assert torch.equal(pb.jacobian(th, big.lam, row0=lo, nrows=cnt, ld=pb.P + 9), J_b[lo:lo + cnt])
 
 
+@pytest.mark.parametrize("name,hidden,n,n_bnd", [
+    ("burgers", [24, 24], 4096, 0), ("ccf", [64, 33, 64], 4100, 0), ("ipm", [64, 27, 64, 40], 2049, 2055),
+    ("boussinesq", [48, 48, 48], 2100, 40)])
+@pytest.mark.parametrize("frozen", [False, True])
+def test_gradient_equals_the_rows(name, hidden, n, n_bnd, frozen):
+    """J^T seed by the adjoint against the same product with the Jacobian's rows: both are FP64 sums of
+    n_rows products, each off by at most n_rows u times the sum of the magnitudes."""
+    big, _, _, pb, _ = _pair(name, hidden, n, n_bnd)
+    pb.gn_set_lambda_trainable(not frozen)
+    th = dev(big.theta)
+    J = pb.jacobian(th, big.lam)
+    seed = dev(np.random.default_rng(2).standard_normal(pb.n_rows))
+    bound = 2.0 ** -53 * 2 * pb.n_rows * (J.abs().T @ seed.abs()) + TOL * (J.abs().T @ seed.abs())
+    assert bool(((pb.gradient(th, big.lam, seed) - J.T @ seed).abs() <= bound).all())
+    r = pb.residual(th, big.lam)[0]
+    g = pb.gradient(th, big.lam)
+    bound = 2.0 ** -53 * 2 * pb.n_rows * (J.abs().T @ r.abs()) + TOL * (J.abs().T @ r.abs())
+    assert bool(((g - J.T @ r).abs() <= bound).all())
+    assert torch.equal(g, pb.gradient(th, big.lam))      # a fixed order of additions
+
+
 def test_many_wall_points_equal_few():
     """2050 wall points take the layered path, 900 of them the pointwise one."""
     big, _, _, pb, _ = _pair("ipm", [32, 32, 32], 300, n_bnd=2050)
