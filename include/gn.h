@@ -83,7 +83,9 @@ enum gn_precision {
   GN_PREC_SPLIT_BF16 = 1,  /* Ozaki split: each FP64 column of J~ scaled by a power of two and
                               split into n_slices BF16 slices; slice products on the tcgen05
                               tensor cores with exactly representable FP32 partial sums,
-                              combined in double-FP32 and returned as FP64 */
+                              combined in double-FP32 and returned as FP64.  With six slices the
+                              Gram takes the same 48-bit operands by their residues modulo 13
+                              coprime numbers instead: the exact integer product, rounded once */
   GN_PREC_SPLIT_ALL = 2    /* as GN_PREC_SPLIT_BF16, and the other two dense contractions too:
                               the CCF Hilbert contraction J_U = K J_g and the trailing updates
                               of the blocked Cholesky factorisation (accumulated in double-FP32;
@@ -216,7 +218,9 @@ int gn_set_precision(gn_handle* h, int precision, int n_slices);
  * keep the launch within four waves of the 152 SMs and at least 256 rows per part) is
  * timed with CUDA events on the handle's stream and the fastest kept for every handle of
  * that shape; the tuning launch synchronises the stream.  ksplit = 1..8 forces a factor.
- * The split changes only the order of the final FP64 additions.  GN_ERR_INVALID otherwise.
+ * The split changes only the order of the final FP64 additions.  With six slices and neither a
+ * split nor a tile forced the Gram goes by residues, which has no split: 1 is reported.
+ * GN_ERR_INVALID otherwise.
  * gn_gram_split_choice reports the factor a Gram over nrows rows uses (0: not tuned yet). */
 int gn_set_gram_split(gn_handle* h, int ksplit);
 int gn_gram_split_choice(const gn_handle* h, int64_t nrows, int* ksplit);

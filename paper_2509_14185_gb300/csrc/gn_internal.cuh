@@ -171,6 +171,7 @@ struct gn_handle {
   int capturing = 0;              // a stream capture is in progress: no workspace may grow
   int lam_frozen = 0;             // lambda held fixed (funnel inference trains at fixed lambda)
   int gram_ksplit = 0;            // split-K factor of the split Gram (0: autotuned per shape)
+  int crt_off = 0;                // the residue planes' workspace could not be allocated
   int gram_tile = 0;              // output tile width of the split Gram, 128 or 64 (0: autotuned)
   // stage 2 of multi-stage training (gn_set_stage1): the stage-1 field jets at every point
   int staged = 0;
@@ -373,6 +374,19 @@ int oz_prepare_cols(int S, const double* X, int64_t ld, int64_t k, int64_t n, co
 // X is n x K row-major (operand row j = row j of X)
 int oz_prepare_rows(int S, const double* X, int64_t ld, int64_t n, int64_t k, const OzOperand& op,
                     cudaStream_t st);
+// e[j] with 2^e > max_k |X_kj| (0 for j >= n), n columns padded to npad; part as above
+int oz_column_exponents(const double* X, int64_t ld, int64_t k, int64_t n, int64_t npad, int* e, double* part,
+                        cudaStream_t st);
+// The six-slice Gram by residues (crt.cu): rows per product, tiles per batch and workspace layout
+struct CrtPlan {
+  int64_t npad, krows, batch, planes, res;
+  size_t bytes;
+};
+CrtPlan crt_plan(int64_t n, int64_t nrows);
+int crt_prepare(const CrtPlan& pl, const double* J, int64_t ld, int64_t k, int64_t n, void* ws, double* part,
+                cudaStream_t st);
+int crt_product(const CrtPlan& pl, int64_t k, int64_t n, void* ws, double* G, int64_t ldg, int add, int64_t tile0,
+                int64_t ntiles, int colmajor, int max_ctas, int* flag, cudaStream_t st);
 // C (M x N, ldc) op= A B^T; sym: only tiles with row tile >= column tile (A must equal B);
 // mode 0: C = v, 1: C += rowscale[i] v (rowscale may be null), 2: C -= v.  flag: bit 1 on timeout.
 // ksplit > 1 (modes 0-2, single exponents only): the contraction is cut into ksplit parts

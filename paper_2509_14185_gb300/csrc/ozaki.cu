@@ -74,17 +74,6 @@ __host__ __device__ constexpr int bar_offset(int S, int BN) {
                                                                 : park_bytes(BN);
 }
 
-// AND of a predicate over the 256 epilogue threads (named barrier 1): every one of them takes
-// the same branch afterwards, so all run the same sequence of named-barrier syncs
-__device__ __forceinline__ bool epilogue_all(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.b32 p, %1, 0;\n bar.red.and.pred q, 1, 256, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r)
-      : "r"((uint32_t)v)
-      : "memory");
-  return r != 0;
-}
 // (hi, lo) += v in double-FP32: TwoSum (Knuth) puts the exact rounding error of
 // hi + v into lo; lo stays ~2^-24 |hi| per add, so no renormalisation is needed
 // before the final (double) hi + (double) lo.  Intrinsics keep the order.
@@ -735,11 +724,8 @@ int encode(const OzOperand& op, int S, CUtensorMap* map, int box_rows = TM) {
 template <int S>
 int prep_cols(const double* X, int64_t ld, int64_t k, int64_t n, const OzOperand& op, double* part,
               cudaStream_t st) {
-  dim3 g((unsigned)((n + 127) / 128), CM_CHUNKS);
-  colmax_partial<<<g, 128, 0, st>>>(X, ld, k, n, part);
-  count_launch();
-  colexp_kernel<<<(unsigned)((op.npad + 255) / 256), 256, 0, st>>>(part, n, op.npad, op.e);
-  count_launch();
+  const int rc = oz_column_exponents(X, ld, k, n, op.npad, op.e, part, st);
+  if (rc) return rc;
   dim3 gs((unsigned)((op.kpad + 63) / 64), (unsigned)(op.npad / 32));   // kpad is a multiple of 32
   split_cols_kernel<S><<<gs, 256, 0, st>>>(X, ld, k, n, op.e, op.npad, op.kpad,
                                           static_cast<__nv_bfloat16*>(op.slices));
@@ -760,6 +746,16 @@ int prep_rows(const double* X, int64_t ld, int64_t n, int64_t k, const OzOperand
 }
 
 }  // namespace
+
+int oz_column_exponents(const double* X, int64_t ld, int64_t k, int64_t n, int64_t npad, int* e, double* part,
+                        cudaStream_t st) {
+  dim3 g((unsigned)((n + 127) / 128), CM_CHUNKS);
+  colmax_partial<<<g, 128, 0, st>>>(X, ld, k, n, part);
+  count_launch();
+  colexp_kernel<<<(unsigned)((npad + 255) / 256), 256, 0, st>>>(part, n, npad, e);
+  count_launch();
+  return GN_NOTE(cudaGetLastError()) == cudaSuccess ? GN_OK : GN_ERR_CUDA;
+}
 
 // Testing hooks of the bounded waits (gn_test_bounded_waits): the bound on every mbarrier wait
 // of the split GEMM, and whether its producer issues no copies.
@@ -1062,12 +1058,44 @@ int gram_tile_choice(int S, int64_t Pp, int64_t nrows) {
   return lookup(S, Pp, nrows, &ch) ? ch.tn : 0;
 }
 
+// Six slices without a forced tile or split go by residues (crt.cu): fewer products, and exact.
+// Not when its workspace could not be had, nor for a wide G of few rows, where writing and
+// reconstructing 13 residues per entry costs more than the products save.  Best slice products /
+// residues in ms: 322 columns, 1025 rows 0.110 / 0.066; 1154, 1025 0.127 / 0.103; 2498, 1025 0.241 / 0.215; 4850, 1025
+// 0.520 / 0.572; 8514, 1025 1.39 / 1.57; 8514, 4097 4.33 / 3.74; 8514, 16385 16.1 / 12.7.
+namespace {
+bool by_residues(const gn_handle* h, int64_t nrows) {
+  return h->n_slices == 6 && h->gram_ksplit == 0 && h->gram_tile == 0 && !h->crt_off && 4 * nrows >= h->Pp;
+}
+size_t colmax_bytes(int64_t Pp) { return (size_t)CM_CHUNKS * rup(Pp, TM) * 8 + 256; }
+size_t residue_bytes(const gn_handle* h, int64_t nrows) {
+  return crt_plan(h->Pp, nrows).bytes + colmax_bytes(h->Pp);
+}
+// the choice the gn_gram_*_choice calls report for a shape that goes by residues
+void record_default_choice(const gn_handle* h, int64_t nrows) {
+  std::lock_guard<std::mutex> g(g_tune_mu);
+  g_tune.emplace(std::make_tuple(h->n_slices, (h->Pp + TM - 1) / TM, gram_chunks(nrows)), GramChoice());
+}
+// false: no memory for the planes (remembered), the slices have to do
+bool residue_ws(gn_handle* h, int64_t nrows) {
+  if (!by_residues(h, nrows)) return false;
+  if (ensure_split_ws(h, residue_bytes(h, nrows)) == GN_OK) return true;
+  cudaGetLastError();
+  h->crt_off = 1;
+  return false;
+}
+}  // namespace
+
 // Tune the Gram of the handle's largest row block ahead of a capture, on a zeroed operand
 // (tensor-core time does not depend on the values).
 int pretune_gram(gn_handle* h) {
   if (h->precision == GN_PREC_FP64 || h->gram_ksplit > 0 || h->gram_tile > 0 || h->n_rows <= 0) return GN_OK;
   const int S = h->n_slices;
   const int64_t nrows = h->jrows;
+  if (by_residues(h, nrows)) {
+    record_default_choice(h, nrows);
+    return GN_OK;
+  }
   GramChoice ks;
   if (lookup(S, h->Pp, nrows, &ks)) return GN_OK;
   const size_t opb = oz_operand_bytes(S, h->Pp, nrows);
@@ -1097,6 +1125,12 @@ int prepare_for_capture(gn_handle* h) {
     const int rc = ensure_chol_ws(h, chol_split_ws_bytes(h->Pp, S));
     if (rc) return rc;
   }
+  if (by_residues(h, h->jrows)) {   // the planes when they can be had, else the slices
+    const size_t planes = residue_bytes(h, h->jrows);
+    if (ensure_split_ws(h, planes > need ? planes : need) == GN_OK) return pretune_gram(h);
+    cudaGetLastError();
+    h->crt_off = 1;
+  }
   const int rc = ensure_split_ws(h, need);
   if (rc) return rc;
   return pretune_gram(h);
@@ -1107,8 +1141,21 @@ int split_gram(gn_handle* h, const double* J, int64_t ld, int64_t nrows, double*
   const int S = h->n_slices;
   if (S < 1 || S > kOzMaxSlices) return GN_ERR_UNSUPPORTED;
   if (nrows <= 0) return GN_OK;
+  if (residue_ws(h, nrows)) {
+    const CrtPlan pl = crt_plan(h->Pp, nrows);
+    double* part = reinterpret_cast<double*>(static_cast<unsigned char*>(h->split_ws) + pl.bytes);
+    for (int64_t k0 = 0; k0 < nrows; k0 += pl.krows) {
+      const int64_t k = k0 + pl.krows < nrows ? pl.krows : nrows - k0;
+      int rc = crt_prepare(pl, J + k0 * ld, ld, k, h->Pp, h->split_ws, part, h->st);
+      if (!rc)
+        rc = crt_product(pl, k, h->Pp, h->split_ws, G, h->Pp, accumulate || k0 > 0, 0, -1, 0, 0, h->flag + 2, h->st);
+      if (rc) return rc;
+    }
+    record_default_choice(h, nrows);
+    return GN_OK;
+  }
   const size_t opb = oz_operand_bytes(S, h->Pp, nrows);
-  const size_t cmb = (size_t)CM_CHUNKS * rup(h->Pp, TM) * 8 + 256;
+  const size_t cmb = colmax_bytes(h->Pp);
   int rc = ensure_split_ws(h, opb + cmb + gram_part_bytes(h->Pp, gram_max_split(h, nrows)));
   if (rc) return rc;
   OzOperand op = oz_operand_at(h->split_ws, S, h->Pp, nrows);
@@ -1141,6 +1188,8 @@ int64_t pipeline_chunk_tiles(gn_handle* h) {
     ch.tn = h->gram_tile > 0 ? h->gram_tile : TN;
   }
   if (ch.ks != 1 || ch.tn != TN) return 0;
+  // the column chunks need every row's residues at once
+  if (by_residues(h, h->n_rows) && crt_plan(h->Pp, h->n_rows).krows < h->n_rows) return 0;
   if ((h->Pp + TM - 1) / TM < 4) return 0;   // a G this small is one strip or two
   if (h->pipe_tiles > 0) return h->pipe_tiles;
   int sms = 0;
@@ -1155,13 +1204,22 @@ int split_gram_pipelined(gn_handle* h, const double* J, int64_t ld, int64_t nrow
   const int S = h->n_slices;
   const int64_t n = h->Pp;
   if (S < 1 || S > kOzMaxSlices || nrows <= 0 || chunk <= 0) return GN_ERR_INVALID;
+  const bool residues = residue_ws(h, nrows);
+  const CrtPlan pl = crt_plan(n, nrows);
   const size_t opb = oz_operand_bytes(S, n, nrows);
-  const size_t cmb = (size_t)CM_CHUNKS * rup(n, TM) * 8 + 256;
-  int rc = ensure_split_ws(h, opb + cmb + gram_part_bytes(n, gram_max_split(h, nrows)));
-  if (rc) return rc;
-  OzOperand op = oz_operand_at(h->split_ws, S, n, nrows);
-  double* part = reinterpret_cast<double*>(static_cast<unsigned char*>(h->split_ws) + opb);
-  rc = oz_prepare_cols(S, J, ld, nrows, n, op, part, st);
+  const size_t cmb = colmax_bytes(n);
+  OzOperand op;
+  int rc = GN_OK;
+  if (residues) {
+    rc = crt_prepare(pl, J, ld, nrows, n, h->split_ws,
+                     reinterpret_cast<double*>(static_cast<unsigned char*>(h->split_ws) + pl.bytes), st);
+  } else {
+    rc = ensure_split_ws(h, opb + cmb + gram_part_bytes(n, gram_max_split(h, nrows)));
+    if (rc) return rc;
+    op = oz_operand_at(h->split_ws, S, n, nrows);
+    rc = oz_prepare_cols(S, J, ld, nrows, n, op,
+                         reinterpret_cast<double*>(static_cast<unsigned char*>(h->split_ws) + opb), st);
+  }
   if (rc) return rc;
   auto new_event = [&](cudaEvent_t* e) -> bool {
     *e = nullptr;
@@ -1173,7 +1231,11 @@ int split_gram_pipelined(gn_handle* h, const double* J, int64_t ld, int64_t nrow
   if (!new_event(&fork) || GN_NOTE(cudaEventRecord(fork, st)) != cudaSuccess ||
       GN_NOTE(cudaStreamWaitEvent(sg, fork, 0)) != cudaSuccess)
     return GN_ERR_CUDA;
-  const int64_t mt = (n + TM - 1) / TM, total = mt * (mt + 1) / 2;
+  // residue tiles are 256 x 256: a quarter of the chunk's tiles per launch, on as many CTAs
+  const int64_t tw = residues ? kCholStrip : TM;
+  const int64_t mt = (n + tw - 1) / tw, total = mt * (mt + 1) / 2;
+  const int max_ctas = (int)(chunk < 2 ? 2 : chunk < (1 << 20) ? chunk : (1 << 20));
+  if (residues) chunk = chunk >= 4 ? chunk / 4 : 1;
   const int64_t nstrip = (n + kCholStrip - 1) / kCholStrip;
   gate.assign((size_t)nstrip, nullptr);
   auto before = [&](int64_t c) { return c * mt - c * (c - 1) / 2; };   // tiles of the columns < c
@@ -1183,10 +1245,11 @@ int split_gram_pipelined(gn_handle* h, const double* J, int64_t ld, int64_t nrow
     rg.tile0 = t0;
     rg.ntiles = (t0 + chunk < total) ? chunk : total - t0;
     rg.colmajor = 1;
-    rc = oz_gemm(S, true, op, op, n, n, G, n, 0, nullptr, h->flag + 2, sg, 1, nullptr, rg);
+    rc = residues ? crt_product(pl, nrows, n, h->split_ws, G, n, 0, rg.tile0, rg.ntiles, 1, max_ctas, h->flag + 2, sg)
+                  : oz_gemm(S, true, op, op, n, n, G, n, 0, nullptr, h->flag + 2, sg, 1, nullptr, rg);
     if (rc) return rc;
     while (tc < mt && before(tc + 1) <= t0 + rg.ntiles) tc++;   // tile columns [0, tc) are done
-    const int64_t sd = (tc * TM >= n) ? nstrip : tc * TM / kCholStrip;   // so are strips [0, sd)
+    const int64_t sd = (tc * tw >= n) ? nstrip : tc * tw / kCholStrip;   // so are strips [0, sd)
     if (sd > strips_done) {
       const int64_t c0 = strips_done * kCholStrip, c1 = (sd * kCholStrip < n) ? sd * kCholStrip : n;
       if (GN_NOTE(add_diag_band(G, A, n, n, c0, c1, gamma, sg)) != cudaSuccess) return GN_ERR_CUDA;
