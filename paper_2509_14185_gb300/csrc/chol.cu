@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(NB * TPR) potrf_inv_kernel(double* A, int64_t 
 }
 
 // Blocked double-float factor of the diagonal block (the split path's critical-path kernel).
-// B = A[k0:k0+kb, k0:k0+kb] - U (lower), scaled B' = D B D by powers of two (D_ii = 2^-sc[i],
+// B = A[k0:k0+kb, k0:k0+kb] - U - D (lower; U and, from the panels since, D: the sums of the updates so far), scaled B' = D B D by powers of two (D_ii = 2^-sc[i],
 // B'_ii in [1, 4)), factored as B' = L' L'^T with L'^{-1} formed alongside.  Writes only
 // double-float results: L' (LDF), L'^{-1} (LinvDF), the scales, and (with fw) the
 // forward-substitution block y_k = L'^{-1} D w_k.  The FP64 copies the triangular solves read
@@ -374,6 +374,7 @@ constexpr size_t kPbSmem = (size_t)(2 * NB * kPbLd + (NB - kPbB) * kPbB + 4 * kP
 
 __global__ void __launch_bounds__(kPbThreads) potrf_blk_kernel(const double* A, int64_t lda, int64_t k0, int kb,
                                                                const float2* __restrict__ U, int64_t ldu,
+                                                               const float2* __restrict__ Dk,
                                                                float2* LDF, float2* LinvDF, int* scOut,
                                                                const double* fw, double* fy, float2* fyDF,
                                                                int* flag) {
@@ -398,8 +399,8 @@ __global__ void __launch_bounds__(kPbThreads) potrf_blk_kernel(const double* A, 
     if (t < kb) {
       double d = A[(k0 + t) * lda + k0 + t];
       if (U) {
-        const float2 u = U[(k0 + t) * ldu + k0 + t];
-        d -= (double)u.x + (double)u.y;
+        const float2 u = U[(k0 + t) * ldu + k0 + t], v = Dk[t * NB + t];
+        d -= ((double)u.x + (double)u.y) + ((double)v.x + (double)v.y);
       }
       if (d > 0.0 && isfinite(d)) e = ilogb(d) >> 1;   // floor(log2(d) / 2)
     }
@@ -410,13 +411,14 @@ __global__ void __launch_bounds__(kPbThreads) potrf_blk_kernel(const double* A, 
   // global loads are all issued before the scales are known
   constexpr int kPer = NB * NB / kPbThreads;
   double av[kPer];
-  float2 uv[kPer];
+  float2 uv[kPer], dv[kPer];
 #pragma unroll
   for (int m = 0; m < kPer; m++) {
     const int idx = t + m * kPbThreads, i = idx / NB, c = idx % NB;
     const bool in = c <= i && i < kb;
     av[m] = in ? A[(k0 + i) * lda + k0 + c] : 0.0;
     uv[m] = (in && U) ? U[(k0 + i) * ldu + k0 + c] : make_float2(0.f, 0.f);
+    dv[m] = (in && U) ? Dk[i * NB + c] : make_float2(0.f, 0.f);
   }
   __syncthreads();
 #pragma unroll
@@ -425,7 +427,8 @@ __global__ void __launch_bounds__(kPbThreads) potrf_blk_kernel(const double* A, 
     if (c > i) continue;
     T v = (i == c) ? AR::one() : AR::zero();
     if (i < kb) {
-      const float2 u = uv[m];
+      const T s = AR::add({uv[m].x, uv[m].y}, {dv[m].x, dv[m].y});
+      const float2 u = make_float2(s.h, s.l);
       v = AR::load_scaled(av[m], U ? &u : nullptr, -(sc[i] + sc[c]));
     }
     S(i, c) = v;
@@ -727,13 +730,21 @@ constexpr int kPanelDFThreads = 256;                       // 16 x 16: 1 row x 4
 constexpr int kPanelDFRowStride = kPanelDFThreads / 16;    // rows ty + 16 a
 constexpr int kPanelDFRows = kPanelDFRowsCTA / kPanelDFRowStride;
 
+// Beside its rows, the panel forms what the next diagonal factors wait for: a cluster of four CTAs
+// holds the 64 rows of one block b below the panel, and the first ndiag clusters add L_b L_b^T (lower) to
+// that block's D (64 x 64 double-float; assigned with dfirst), the rows exchanged through
+// distributed shared memory.  So the factor of the next block follows the panel directly, while the tensor-core
+// update of the rows below it (17-31 us) runs beside that factor instead of before it.  At n = 1154 the panel takes
+// 17.5 us instead of 11.3 (two cluster barriers and the exchange 3 us, the sums 3 us with two entries a thread; 8 us when
+// a thread had four of one row).
 template <int S>
-__global__ void __launch_bounds__(kPanelDFThreads) panel_df_kernel(double* A, int64_t lda, int64_t k0, int kb, int64_t k1,
+__global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kPanelDFThreads) panel_df_kernel(double* A, int64_t lda, int64_t k0, int kb, int64_t k1,
                                                        int64_t n, const float2* __restrict__ U, int64_t ldu,
                                                        const float2* __restrict__ LkDF, const int* __restrict__ sck,
                                                        __nv_bfloat16* slices, int* eout, int64_t row_base,
                                                        int64_t npad, int64_t kpad, int kofs,
-                                                       const float2* __restrict__ fyDF, double* fw, const int* flag) {
+                                                       const float2* __restrict__ fyDF, double* fw, float2* D,
+                                                       int ndiag, int dfirst, const int* flag) {
   extern __shared__ __align__(16) unsigned char smraw[];
   float2 (*As)[NB + 1] = reinterpret_cast<float2 (*)[NB + 1]>(smraw);
   float2 (*Lt)[NB + 1] = As + kPanelDFRowsCTA;   // Lt[q][j] = L'^{-1}[j][q]
@@ -885,6 +896,56 @@ __global__ void __launch_bounds__(kPanelDFThreads) panel_df_kernel(double* A, in
       oz_digits<S>(x, e, slices + (r - row_base) * kpad + kofs + j, npad * kpad);
     }
   }
+  const int cl = blockIdx.x >> 2, rank = blockIdx.x & 3;
+  if (cl >= ndiag) return;   // the same for the whole cluster
+  static_assert(kPanelDFRows == 1 && kPanelDFRowsCTA * 4 == NB, "a cluster holds one block's rows");
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < 4; b++) As[ty][tx + 16 * b] = make_float2(ah[0][b], al[0][b]);
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  float2 in[NB * NB / kPanelDFThreads];   // all loads in flight before the first is stored
+#pragma unroll
+  for (int m = 0; m < NB * NB / kPanelDFThreads; m++) {   // row r of the block: CTA r / 16
+    const int r = (t + m * kPanelDFThreads) / NB, c = t % NB;
+    const uint32_t addr = static_cast<uint32_t>(__cvta_generic_to_shared(&As[r & 15][c]));
+    asm volatile("{\n .reg .u32 a;\n mapa.shared::cluster.u32 a, %2, %3;\n ld.shared::cluster.v2.f32 {%0, %1}, [a];\n}\n"
+                 : "=f"(in[m].x), "=f"(in[m].y)
+                 : "r"(addr), "r"(r >> 4));
+  }
+#pragma unroll
+  for (int m = 0; m < NB * NB / kPanelDFThreads; m++) Lt[(t + m * kPanelDFThreads) / NB][t % NB] = in[m];
+  // (also: no CTA leaves while another still reads its rows)
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  // the 2080 lower entries dealt out over the cluster's 1024 threads, two each; every sum runs in two
+  // interleaved halves
+  float2* Db = D + (int64_t)cl * NB * NB;
+  for (int o = rank * kPanelDFThreads + t; o < NB * (NB + 1) / 2; o += 4 * kPanelDFThreads) {
+    int i = (int)((sqrtf(8.0f * (float)o + 1.0f) - 1.0f) * 0.5f);
+    while ((i + 1) * (i + 2) / 2 <= o) i++;
+    while (i * (i + 1) / 2 > o) i--;
+    const int c = o - i * (i + 1) / 2;
+    float dh[2] = {0.f, 0.f}, dl[2] = {0.f, 0.f};
+#pragma unroll 4
+    for (int q = 0; q < NB; q += 2)
+#pragma unroll
+      for (int z = 0; z < 2; z++) {
+        const float2 x = Lt[i][q + z], y = Lt[c][q + z];
+        const float p = __fmul_rn(x.x, y.x);
+        float pe = __fmaf_rn(x.x, y.x, -p);
+        pe = __fmaf_rn(x.x, y.y, __fmaf_rn(x.y, y.x, pe));
+        const float s1 = __fadd_rn(dh[z], p);
+        const float bb = __fsub_rn(s1, dh[z]);
+        const float err = __fadd_rn(__fsub_rn(dh[z], __fsub_rn(s1, bb)), __fsub_rn(p, bb));
+        dh[z] = s1;
+        dl[z] = __fadd_rn(dl[z], __fadd_rn(pe, err));
+      }
+    DF v = ArithDF::add({dh[0], dl[0]}, {dh[1], dl[1]});
+    if (!dfirst) {
+      const float2 old = Db[i * NB + c];
+      v = ArithDF::add({old.x, old.y}, v);
+    }
+    Db[i * NB + c] = make_float2(v.h, v.l);
+  }
 }
 
 // Blocked triangular solves with the stored diagonal inverses.  One launch per
@@ -982,11 +1043,11 @@ cudaError_t launch_potrf(double* A, int64_t lda, int64_t k0, int kb, const float
 }
 
 cudaError_t launch_potrf_blk(const double* A, int64_t lda, int64_t k0, int kb, const float2* U, int64_t ldu,
-                             float2* LDF, float2* LinvDF, int* scOut, const double* fw, double* fy, float2* fyDF,
+                             const float2* Dk, float2* LDF, float2* LinvDF, int* scOut, const double* fw, double* fy, float2* fyDF,
                              int* flag, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(potrf_blk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPbSmem);
   if (e != cudaSuccess) return e;
-  potrf_blk_kernel<<<1, kPbThreads, kPbSmem, st>>>(A, lda, k0, kb, U, ldu, LDF, LinvDF, scOut, fw, fy, fyDF, flag);
+  potrf_blk_kernel<<<1, kPbThreads, kPbSmem, st>>>(A, lda, k0, kb, U, ldu, Dk, LDF, LinvDF, scOut, fw, fy, fyDF, flag);
   count_launch();
   return cudaGetLastError();
 }
@@ -1016,30 +1077,30 @@ cudaError_t launch_panel(double* A, int64_t lda, int64_t k0, int kb, int64_t k1,
 template <int S>
 cudaError_t launch_panel_df(double* A, int64_t lda, int64_t k0, int kb, int64_t k1, int64_t n, const float2* U,
                             int64_t ldu, const float2* LkDF, const int* sck, const OzOperand& op, int* eout,
-                            int64_t row_base, int kofs, const float2* fyDF, double* fw, const int* flag,
-                            cudaStream_t st) {
+                            int64_t row_base, int kofs, const float2* fyDF, double* fw, float2* D, int ndiag,
+                            int dfirst, const int* flag, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(panel_df_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kPanelDFSmem);
   if (e != cudaSuccess) return e;
-  const int64_t blocks = (n - k1 + kPanelDFRowsCTA - 1) / kPanelDFRowsCTA;
+  const int64_t blocks = (n - k1 + NB - 1) / NB * 4;   // whole clusters
   if (blocks <= 0) return cudaSuccess;
   panel_df_kernel<S><<<(unsigned)blocks, kPanelDFThreads, kPanelDFSmem, st>>>(A, lda, k0, kb, k1, n, U, ldu, LkDF, sck,
                                                                   static_cast<__nv_bfloat16*>(op.slices), eout,
-                                                                  row_base, op.npad, op.kpad, kofs, fyDF, fw,
-                                                                  flag);
+                                                                  row_base, op.npad, op.kpad, kofs, fyDF, fw, D, ndiag,
+                                                                  dfirst, flag);
   count_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_panel_split(int S, double* A, int64_t lda, int64_t k0, int kb, int64_t k1, int64_t n,
                                const float2* U, int64_t ldu, const float2* LkDF, const int* sck, const OzOperand& op,
-                               int* eout, int64_t row_base, int kofs, const float2* fyDF, double* fw,
-                               const int* flag, cudaStream_t st) {
+                               int* eout, int64_t row_base, int kofs, const float2* fyDF, double* fw, float2* D,
+                               int ndiag, int dfirst, const int* flag, cudaStream_t st) {
   switch (S) {
 #define GN_PANEL_CASE(s)                                                                                   \
   case s:                                                                                                  \
     return launch_panel_df<s>(A, lda, k0, kb, k1, n, U, ldu, LkDF, sck, op, eout, row_base, kofs, fyDF, fw, \
-                              flag, st);
+                              D, ndiag, dfirst, flag, st);
     GN_PANEL_CASE(1)
     GN_PANEL_CASE(2)
     GN_PANEL_CASE(3)
@@ -1116,10 +1177,15 @@ cudaError_t cholesky_factor(gn_handle* h, double* A, int64_t n, int64_t lda, dou
 // columns first get the updates of the strip's earlier panels (a 64-column
 // split GEMM over the chunks already written).
 //
-// Look-ahead: the bulk update of strip t is split into the next strip's 256
-// columns, done at once on the critical stream, and the rest, deferred to a
-// low-priority stream where it overlaps strip t + 1's chain (which touches only
-// its own columns).  Strip operands alternate between two buffers.
+// Three streams.  The critical one holds only diagonal factors and panels: a factor needs of the updates
+// no more than its own 64 x 64 block, which the panels before it form on the CUDA cores (D, panel_df_kernel), so
+// it follows the panel directly.  The updates of the columns below it run on a second stream beside it
+// and are waited for by its panel: inside the strip, the next block's columns; at its end, the next
+// strip's 256 columns.  The rest of the strip's bulk update is deferred to a low-priority stream, where it
+// overlaps the next strip's chain.  Strip operands alternate between two buffers.  Damped solve against
+// updates in line with the factors: n = 98 0.160 -> 0.147 ms, 482 0.652 -> 0.537, 1154 1.557 -> 1.274, 4850 7.08 -> 6.03,
+// 8514 16.7 -> 15.4, 12674 39.1 -> 37.4 (from a few thousand columns the bulk updates' tensor time sets the pace;
+// 128 x 64 tiles for them, which would free SMs sooner, took 16.6 ms at 8514).
 //
 // The diagonal blocks and the panels are computed in double-float arithmetic
 // (about 48 significant bits, the precision U and the split GEMM carry).
@@ -1130,8 +1196,8 @@ cudaError_t cholesky_factor(gn_handle* h, double* A, int64_t n, int64_t lda, dou
 constexpr int64_t kStrip = kCholStrip;
 
 // Split workspace of cholesky_factor_split: U (n x n double-FP32), two strip operands
-// (slices and four exponent arrays each), the double-float diagonal factors and inverses, their
-// scales and the double-float forward-solve block.
+// (slices and four exponent arrays each), the double-float diagonal factors, inverses and
+// updates D, the scales and the double-float forward-solve block.
 size_t chol_split_ws_bytes(int64_t n, int S) {
   auto rup = [](int64_t v, int64_t m) { return (v + m - 1) / m * m; };
   const int64_t npad0 = rup(n, 128);
@@ -1143,22 +1209,28 @@ size_t chol_split_ws_bytes(int64_t n, int S) {
   const size_t lb = rup(nblk * NB * NB * sizeof(float2), 256);
   const size_t cb = rup(nblk * NB * sizeof(int), 256);
   const size_t yb = rup(NB * sizeof(float2), 256);
-  return ub + 2 * (sb + eb) + 2 * lb + cb + yb + 256;
+  return ub + 2 * (sb + eb) + 3 * lb + cb + yb + 256;
 }
 
-// The look-ahead's streams: the critical path at the highest priority, the deferred bulk
-// updates in the middle, and the pipelined step's Gram chunks at the lowest (numerically
-// greater is lower; with only two levels the last two share one).
+// The look-ahead's streams: the critical path at the highest priority, the updates of the next
+// columns below it (a diagonal factor needs an SM to itself, so it must not find them all taken),
+// the deferred bulk updates in the middle, and the pipelined step's Gram chunks at the lowest
+// (numerically greater is lower; with fewer levels neighbours share one).
 cudaError_t ensure_chol_streams(gn_handle* h) {
   if (h->st_hi) return cudaSuccess;
   int least = 0, greatest = 0;
   cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
   const int middle = greatest + (least - greatest + 1) / 2;
+  const int next = greatest < middle ? greatest + 1 : greatest;
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_hi, cudaStreamNonBlocking, greatest);
+  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_up, cudaStreamNonBlocking, next);
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_lo, cudaStreamNonBlocking, middle);
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_g, cudaStreamNonBlocking, least);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_panel, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_rest, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_next, cudaEventDisableTiming);
+  for (cudaEvent_t& b : h->ev_bulk)
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b, cudaEventDisableTiming);
   return e;
 }
 
@@ -1205,106 +1277,128 @@ cudaError_t cholesky_factor_split(gn_handle* h, double* A, int64_t n, int64_t ld
     const cudaError_t e = ensure_chol_streams(h);
     if (e != cudaSuccess) return e;
   }
-  cudaStream_t sh = h->st_hi, sl = h->st_lo;
+  float2* D = reinterpret_cast<float2*>(reinterpret_cast<unsigned char*>(LDF) + lb);
+  cudaStream_t sh = h->st_hi, su = h->st_up, sl = h->st_lo;
   const int64_t nstrip = (n + kStrip - 1) / kStrip;
-  std::vector<cudaEvent_t> evs(2 * nstrip + 3, nullptr);
   cudaError_t err = cudaSuccess;
-  for (auto& e : evs)
-    if (err == cudaSuccess) err = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
-  struct Guard {   // events may be destroyed while work on them is pending
-    std::vector<cudaEvent_t>& v;
-    ~Guard() {
-      for (auto e : v)
-        if (e) cudaEventDestroy(e);
-    }
-  } guard{evs};
-  if (err != cudaSuccess) return err;
-  cudaEvent_t* evA = evs.data();            // [t]: strip t's next-columns update done
-  cudaEvent_t* evB = evs.data() + nstrip;   // [t]: strip t's deferred bulk update done
-  cudaEvent_t e0 = evs[2 * nstrip], e_hi = evs[2 * nstrip + 1], e_lo = evs[2 * nstrip + 2];
-  std::vector<char> launchedB(nstrip, 0);
   auto fail = [&](int code) {
     *rc_out = code;
     return cudaErrorUnknown;
   };
-  if ((err = cudaEventRecord(e0, st)) != cudaSuccess) return err;
-  if ((err = cudaStreamWaitEvent(sh, e0, 0)) != cudaSuccess) return err;
-  if ((err = cudaStreamWaitEvent(sl, e0, 0)) != cudaSuccess) return err;
-  if ((err = cudaMemsetAsync(U, 0, (size_t)n * n * sizeof(float2), sh)) != cudaSuccess) return err;
-  if (b && (err = cudaMemcpyAsync(w, b, n * sizeof(double), cudaMemcpyDeviceToDevice, sh)) != cudaSuccess) return err;
+  auto record = [&](cudaEvent_t e, cudaStream_t s) {
+    if (err == cudaSuccess) err = cudaEventRecord(e, s);
+  };
+  auto wait = [&](cudaStream_t s, cudaEvent_t e) {
+    if (err == cudaSuccess) err = cudaStreamWaitEvent(s, e, 0);
+  };
+  // U[r0:, c0:c0+nc] += L[r0:, s0:s0+kuse] L[c0:c0+nc, s0:s0+kuse]^T from the strip's operand (128 x 64 tiles)
+  auto update = [&](const OzOperand& strip, int64_t s0, int64_t r0, int64_t c0, int64_t nc, int64_t kuse) {
+    OzOperand va = oz_operand_rows(strip, S, r0 - s0), vb = oz_operand_rows(strip, S, c0 - s0);
+    va.kuse = vb.kuse = kuse;
+    return oz_gemm(S, false, va, vb, n - r0, nc, reinterpret_cast<double*>(U + r0 * n + c0), n, 3, nullptr,
+                   h->flag + 2, su, 1, nullptr, OzRange(), 64);
+  };
+  // (events are recorded again for every block: a wait is on the record before it)
+  cudaEvent_t eP = h->ev_panel, eU = h->ev_rest, eN = h->ev_next, *eB = h->ev_bulk;
+  record(eP, st);
+  wait(sh, eP);
+  wait(su, eP);
+  wait(sl, eP);
+  if (err == cudaSuccess) err = cudaMemsetAsync(U, 0, (size_t)n * n * sizeof(float2), sh);
+  if (b && err == cudaSuccess) err = cudaMemcpyAsync(w, b, n * sizeof(double), cudaMemcpyDeviceToDevice, sh);
+  if (err != cudaSuccess) return err;
   cudaEvent_t waited = nullptr;
   for (int64_t t = 0; t < nstrip; t++) {
     const int64_t s0 = t * kStrip;
     const int64_t s1 = (s0 + kStrip < n) ? s0 + kStrip : n;
     // the strip's columns of A may still be in production (pipelined step)
     if (gate && gate[t] && gate[t] != waited) {
-      if ((err = cudaStreamWaitEvent(sh, gate[t], 0)) != cudaSuccess) return err;
+      wait(sh, gate[t]);
       waited = gate[t];
     }
-    // strip operand t % 2 (rows relative to s0); its previous user, strip t - 2's deferred
-    // update, finished before strip t - 1's next-columns update (the wait below)
+    // The first factor reads U of the strips before t - 1 (strip t - 1's share is in D): their
+    // deferred updates end with strip t - 2's.  That was also the last user of strip operand t % 2.
+    if (t >= 2) wait(sh, eB[t & 1]);
     unsigned char* sbase = strip_base + (t & 1) * (sb + eb);
-    OzOperand strip;
+    OzOperand strip;   // rows relative to s0
     strip.slices = sbase;
     strip.e = reinterpret_cast<int*>(sbase + sb);
     strip.npad = rup(n - s0, 128);
     strip.kpad = kStrip;
     strip.echunk = NB;
     strip.estride = estride;
-    // the strip's chain: in-strip updates, diagonal factors, panels
     for (int64_t k0 = s0; k0 < s1; k0 += NB) {
       const int kb = (int)((n - k0) < NB ? (n - k0) : NB);
-      const int kofs = (int)(k0 - s0);
-      if (kofs > 0) {
-        // U[k0:, k0:k0+kb] += L[k0:, s0:k0] L[k0:k0+kb, s0:k0]^T (64 columns: 128 x 64 tiles)
-        OzOperand v = oz_operand_rows(strip, S, k0 - s0);
-        v.kuse = kofs;
-        rc = oz_gemm(S, false, v, v, n - k0, kb, reinterpret_cast<double*>(U + k0 * n + k0), n, 3, nullptr,
-                     h->flag + 2, sh, 1, nullptr, OzRange(), 64);
-        if (rc) return fail(rc);
-      }
+      const int kofs = (int)(k0 - s0), j = kofs / NB;
+      // blocks 1 .. 3 of the strip: U of their diagonal comes with strip t - 1's update of the strip
+      if (j == 1 && t > 0) wait(sh, eN);
+      if (err != cudaSuccess) return err;
       const float2* Uk = (k0 > 0) ? U : nullptr;
-      err = launch_potrf_blk(A, lda, k0, kb, Uk, n, LDF, LinvDF, scales, b ? w : nullptr, y, yDF, flag, sh);
+      err = launch_potrf_blk(A, lda, k0, kb, Uk, n, D + (k0 / NB) * NB * NB, LDF, LinvDF, scales, b ? w : nullptr, y,
+                             yDF, flag, sh);
       if (err != cudaSuccess) return err;
       const int64_t k1 = k0 + kb;
       if (k1 >= n) break;
-      err = launch_panel_split(S, A, lda, k0, kb, k1, n, Uk, n, LinvDF + (k0 / NB) * NB * NB,
-                               scales + (k0 / NB) * NB, strip, strip.e + (kofs / NB) * estride, s0, kofs, yDF,
-                               b ? w : nullptr, flag, sh);
+      // the rows below: their update from the strip's earlier panels, or from the strip before (j = 0)
+      if (j > 0 || t > 0) wait(sh, eU);
       if (err != cudaSuccess) return err;
+      // D of the strip's blocks below and of the next strip's first one
+      err = launch_panel_split(S, A, lda, k0, kb, k1, n, Uk, n, LinvDF + (k0 / NB) * NB * NB,
+                               scales + (k0 / NB) * NB, strip, strip.e + j * estride, s0, kofs, yDF,
+                               b ? w : nullptr, D + (k1 / NB) * NB * NB, (int)(kStrip / NB) - j, j == 0 ? 1 : 0, flag,
+                               sh);
+      if (err != cudaSuccess) return err;
+      record(eP, sh);
+      wait(su, eP);
+      // the next block's columns below its diagonal, beside its factor
+      if (k1 < s1 && k1 + NB < n) {
+        rc = update(strip, s0, k1 + NB, k1, NB, kofs + NB);
+        if (rc) return fail(rc);
+      }
+      if (k1 < s1) record(eU, su);
     }
+    if (err != cudaSuccess) return err;
     if (s1 >= n) break;
-    // bulk update of the trailing matrix, U[s1:, s1:] += L[s1:, s0:s1] L[s1:, s0:s1]^T
-    OzOperand wb = oz_operand_rows(strip, S, s1 - s0);
-    // (a) the next strip's columns now, on the critical path; the deferred update of strip
-    //     t - 1 writes those columns too, so it must be done first
-    if (t >= 1 && launchedB[t - 1] && (err = cudaStreamWaitEvent(sh, evB[t - 1], 0)) != cudaSuccess) return err;
-    const int64_t nn = (n - s1 < kStrip) ? n - s1 : kStrip;
-    rc = oz_gemm(S, false, wb, wb, n - s1, nn, reinterpret_cast<double*>(U + s1 * n + s1), n, 3, nullptr,
-                 h->flag + 2, sh, 1, nullptr, OzRange(), 64);
-    if (rc) return fail(rc);
-    if ((err = cudaEventRecord(evA[t], sh)) != cudaSuccess) return err;
+    // The trailing matrix, U[s1:, s1:] += L[s1:, s0:s1] L[s1:, s0:s1]^T.  (a) the next strip's columns at
+    // once: first its first block's below the diagonal (its panel waits for them), then the rest
+    // below that block's rows.  Strip t - 1's deferred update writes those columns too.
+    if (t >= 1) wait(su, eB[(t - 1) & 1]);
+    if (err != cudaSuccess) return err;
+    const int64_t s2 = s1 + kStrip < n ? s1 + kStrip : n, s1b = s1 + NB;
+    if (s1b < n) {
+      rc = update(strip, s0, s1b, s1, NB, kStrip);
+      if (rc) return fail(rc);
+    }
+    record(eU, su);
+    if (s1b < n) {
+      rc = update(strip, s0, s1b, s1b, s2 - s1b, kStrip);
+      if (rc) return fail(rc);
+    }
+    record(eN, su);
     // (b) the rest, U[s2:, s2:] (lower tiles), deferred to sl: it overlaps the next strip's
     //     chain, which touches only the next strip's columns
-    const int64_t s2 = s1 + kStrip;
     if (s2 < n) {
-      if ((err = cudaStreamWaitEvent(sl, evA[t], 0)) != cudaSuccess) return err;
-      OzOperand wv = oz_operand_rows(wb, S, kStrip);
+      wait(sl, eN);
+      if (err != cudaSuccess) return err;
+      OzOperand wv = oz_operand_rows(strip, S, s2 - s0);
       rc = oz_gemm(S, true, wv, wv, n - s2, n - s2, reinterpret_cast<double*>(U + s2 * n + s2), n, 3, nullptr,
                    h->flag + 2, sl);
       if (rc) return fail(rc);
-      if ((err = cudaEventRecord(evB[t], sl)) != cudaSuccess) return err;
-      launchedB[t] = 1;
     }
+    record(eB[t & 1], sl);
   }
+  if (err != cudaSuccess) return err;
   // the FP64 copies of the diagonal blocks' factors for the triangular solves
   diag_to_fp64_kernel<<<(unsigned)nblk, 256, 0, sh>>>(A, lda, n, LDF, LinvDF, scales, Linv, flag);
   count_launch();
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  if ((err = cudaEventRecord(e_hi, sh)) != cudaSuccess) return err;
-  if ((err = cudaEventRecord(e_lo, sl)) != cudaSuccess) return err;
-  if ((err = cudaStreamWaitEvent(st, e_hi, 0)) != cudaSuccess) return err;
-  return cudaStreamWaitEvent(st, e_lo, 0);
+  record(eP, sh);
+  record(eU, su);
+  record(eN, sl);
+  wait(st, eP);
+  wait(st, eU);
+  wait(st, eN);
+  return err;
 }
 
 namespace {

@@ -680,10 +680,12 @@ int gn_destroy(gn_handle* h) {
   cudaStreamSynchronize(h->st);
   graph_release(h);
   if (h->st_hi) cudaStreamDestroy(h->st_hi);
+  if (h->st_up) cudaStreamDestroy(h->st_up);
   if (h->st_lo) cudaStreamDestroy(h->st_lo);
   if (h->st_g) cudaStreamDestroy(h->st_g);
   if (h->ev_panel) cudaEventDestroy(h->ev_panel);
-  if (h->ev_rest) cudaEventDestroy(h->ev_rest);
+  for (cudaEvent_t e : {h->ev_rest, h->ev_next, h->ev_bulk[0], h->ev_bulk[1]})
+    if (e) cudaEventDestroy(e);
   destroy_side(h);
   free_all(h);
   if (h->tmaps) free(h->tmaps);

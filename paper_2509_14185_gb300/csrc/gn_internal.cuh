@@ -151,9 +151,10 @@ struct gn_handle {
   int64_t ema_len = 0;
   // streams of the factorisations' look-ahead (created on first use)
   cudaStream_t st_hi = nullptr;   // critical path (highest priority)
+  cudaStream_t st_up = nullptr;   // updates of the next columns (next priority)
   cudaStream_t st_lo = nullptr;   // deferred bulk updates (middle priority)
   cudaStream_t st_g = nullptr;    // Gram chunks of the pipelined step (lowest priority)
-  cudaEvent_t ev_panel = nullptr, ev_rest = nullptr;   // the FP64 factorisation's look-ahead
+  cudaEvent_t ev_panel = nullptr, ev_rest = nullptr, ev_next = nullptr, ev_bulk[2] = {nullptr, nullptr};
   // side stream of the wall and normalisation passes (residual and Jacobian modes), with the
   // events that fork it from and join it to the handle's stream
   cudaStream_t st_aux = nullptr;
