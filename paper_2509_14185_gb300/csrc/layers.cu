@@ -52,6 +52,7 @@ struct LayArgs {
   const double* zin;        // [point][cz][K]: preactivation jets of the producing layer, without its bias
   const double* bias;       // forward: of the producing layer
   double* hout;             // forward: [point][CR][K] activation jets (null: not kept)
+  int* hexp;                // forward: [point][CR] exponents of those rows (with hout)
   const double* hin;        // reverse: the same, of the layer the adjoint passes
   const double* seeds;      // reverse from the outputs: [item][nf][CR]
   const double* Wlast;      // [nf][K]
@@ -358,7 +359,10 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
       for (int c = 0; c < C; c++) {
         const int row = it * C + c;
         const int e = row_exponent(__reduce_max_sync(0xffffffffu, m[c]));
-        if (lane == 0) eA[row] = e;
+        if (lane == 0) {
+          eA[row] = e;
+          if (kFwd && c < CR && p.hexp) p.hexp[pt * CR + c] = e;
+        }
 #pragma unroll
         for (int s = 0; s < 2; s++) {
           if (s < ks_n) {
@@ -413,11 +417,10 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
         uint32_t r[kLayS][8];
 #pragma unroll
         for (int s = 0; s < kLayS; s++)
-          asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                       : "=r"(r[s][0]), "=r"(r[s][1]), "=r"(r[s][2]), "=r"(r[s][3]), "=r"(r[s][4]), "=r"(r[s][5]),
-                         "=r"(r[s][6]), "=r"(r[s][7])
-                       : "r"(tmem + ((uint32_t)((warp & 3) * 32) << 16) + s * kLayW + col0));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          tmem_ld8_async(tmem + ((uint32_t)((warp & 3) * 32) << 16) + s * kLayW + col0, r[s]);
+        tmem_wait_ld();
+#pragma unroll
+        for (int s = 0; s < kLayS; s++) tmem_use8(r[s]);
 #pragma unroll
         for (int j = 0; j < 8; j++) {
           const int col = col0 + j;
@@ -622,8 +625,12 @@ struct LayEntries {
   const double* qb;
   const double* H[GN_MAX_LAYERS + 1];      // [point][CR][w_j], j = 1 .. L - 1
   const double* Ab[GN_MAX_LAYERS + 1];     // [item][CR][w_j]
+  const int* He[GN_MAX_LAYERS + 1];        // [point][CR] exponents of H's rows, j = 1 .. L - 2
   const double* seeds;                     // [item][NF][CR]
   double* J;
+  int hidden;                              // 0: the hidden-to-hidden weights are lay_hidden_entries'
+  int* flag;
+  unsigned long long wait_ns;
 };
 // One warp per (point, layer): the layer's activation jets stay in registers (two neurons per
 // lane) for all rows of the point, the adjoints are read at one address per warp, consecutive lanes
@@ -661,7 +668,7 @@ __global__ void __launch_bounds__(256) lay_entries(const LayEntries p) {
         Jw[o * D] = fma(a0, q, ab[out + o]);
         if constexpr (D == 2) Jw[o * D + 1] = fma(a0, beta, ab[2 * out + o]);
       }
-    } else {
+    } else if (l == L - 1 || p.hidden) {
 #pragma unroll 4
       for (int o = 0; o < out; o++) {
         double v0 = 0.0, v1 = 0.0;
@@ -676,6 +683,191 @@ __global__ void __launch_bounds__(256) lay_entries(const LayEntries p) {
       }
     }
     for (int o = lane; o < out; o += 32) Jb[o] = ab[o * os];
+  }
+}
+
+// Hidden-to-hidden weights of 2D rows as products: sum_c abar_c[o] h_c[i] over the six components is a
+// (rows x out) x 6 x in contraction per point and layer, whose FP64 form (lay_entries) bounds the 2D
+// Jacobian.  One CTA per SM, persistent over (point, layer, pair of rows): 128 x 64 outputs, K = 6 of 16.
+// A component's scale moves between the factors by powers of two (h_c is taken relative to its own
+// largest element 2^eh_c, abar_c times that); then every output row and column has one exponent over
+// its six terms.  62-bit integers in eight digits (nine bits below FP64's last for the row's largest
+// term), the 36 digit pairs of the eight leading levels summed exactly: an entry's error stays below
+// that of the FP64 sum unless all its terms lie 2^9 under the product of its row's and its column's largest.
+// Bound by the digits and the 64-bit recombination (integer pipes) and by J's stores.
+// Jacobian of 32,768 IPM rows, four hidden layers of 64: 6.96 -> 5.54 ms.  Digits dealt over all threads
+// (5.64 ms) and stores of the unit before beside the products (5.67 ms) were no faster.
+constexpr int kEntS = 8;
+constexpr int kEntASlice = 128 * 64, kEntBSlice = 64 * 64;   // K padded to 32: the layout of lay_gemm
+constexpr int kEntOps = kEntS * (kEntASlice + kEntBSlice);
+constexpr size_t kEntSmem = 1024 + kEntOps + 128 * 65 * 8;
+// digits of x 2^(62 - e): bytes 0..6 plus 128, then the signed top
+__device__ __forceinline__ long long biased_digits62(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+  if (ex > 0) m |= 1ull << 52;
+  const int sh = (ex > 0 ? ex : 1) - 1013 - e;   // <= 9
+  unsigned long long v;
+  if (sh >= 0) v = sh > 9 ? 0ull : m << sh;
+  else v = sh < -54 ? 0ull : (m + (1ull << (-sh - 1))) >> -sh;
+  return ((b >> 63) ? -(long long)v : (long long)v) + 0x80808080808080ll;
+}
+__device__ __forceinline__ unsigned short digit62_bf16(long long u, int q) {
+  const unsigned lo = (unsigned)u, hi = (unsigned)((unsigned long long)u >> 32);
+  float f;
+  if (q == 0) f = (float)((int)hi >> 24);
+  else {
+    const int byte = 7 - q;   // 0..6
+    f = __uint_as_float(__byte_perm(byte < 4 ? lo : hi, 0x4B000000u, 0x7540 + (byte & 3))) - 8388736.0f;
+  }
+  return (unsigned short)(__float_as_uint(f) >> 16);
+}
+__global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEntries p) {
+  constexpr int CR = 6;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* As =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  unsigned char* Bs = As + kEntS * kEntASlice;
+  double* out_tile = reinterpret_cast<double*>(As + kEntOps);   // [128][65]
+  __shared__ uint64_t done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int eA[128], eB[64];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  for (int idx = t; idx < kEntOps / 16; idx += kLayThreads)   // components 6 .. 31 stay zero
+    reinterpret_cast<uint4*>(As)[idx] = make_uint4(0, 0, 0, 0);
+  if (t == 0) {
+    mbar_init(&done, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "n"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  const int nl = p.net.L - 2, ng = (p.nr + 1) / 2;
+  const int64_t units = p.npt * nl * ng;
+  // this thread's operand row of a unit (threads 0 .. 127: A row = (row of the pair, o); 128 .. 191:
+  // B row = i), loaded a unit ahead
+  double x[CR];
+  int eh[CR];
+  auto load = [&](int64_t u) {
+#pragma unroll
+    for (int c = 0; c < CR; c++) {
+      x[c] = 0.0;
+      eh[c] = 0;
+    }
+    if (u >= units || t >= 192) return;
+    const int64_t pl = u / (nl * ng);
+    const int l = 1 + (int)(u / ng % nl), g = (int)(u % ng);
+    const int in = p.net.w[l], out = p.net.w[l + 1];
+#pragma unroll
+    for (int c = 0; c < CR; c++) eh[c] = p.He[l][pl * CR + c];
+    if (t < 128) {
+      const int e = 2 * g + (t >> 6), o = t & 63;
+      if (e < p.nr && o < out)
+#pragma unroll
+        for (int c = 0; c < CR; c++) x[c] = p.Ab[l + 1][((pl * p.nr + e) * CR + c) * out + o];
+    } else {
+      const int i = t - 128;
+      if (i < in)
+#pragma unroll
+        for (int c = 0; c < CR; c++) x[c] = p.H[l][(pl * CR + c) * in + i];
+    }
+  };
+  load(blockIdx.x);
+  uint32_t phase = 0;
+  for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+    const int64_t pl = u / (nl * ng);
+    const int l = 1 + (int)(u / ng % nl), g = (int)(u % ng);
+    const int in = p.net.w[l], out = p.net.w[l + 1];
+    if (t < 192) {
+      int m = -100000;
+      bool bad = false;
+#pragma unroll
+      for (int c = 0; c < CR; c++) {
+        const int ex = (int)(abs_hi(x[c]) >> 20);
+        bad = bad || ex == 0x7ff || eh[c] == kLayBad;
+        const int e = (ex > 0 ? ex : 1) - 1022 + (t < 128 ? eh[c] : -eh[c]);
+        if (x[c] != 0.0) m = e > m ? e : m;
+      }
+      if (m == -100000) m = 0;
+      if (t < 128) eA[t] = bad ? kLayBad : m;
+      else eB[t - 128] = bad ? kLayBad : m;
+      unsigned char* row = t < 128 ? As : Bs;
+      const int r = t < 128 ? t : t - 128, stride = t < 128 ? kEntASlice : kEntBSlice;
+#pragma unroll
+      for (int c = 0; c < CR; c++) {
+        const long long v = biased_digits62(x[c], bad ? 5000 : m - (t < 128 ? eh[c] : -eh[c]));
+        unsigned char* dst = row + swz(r, c, 0);
+#pragma unroll
+        for (int d = 0; d < kEntS; d++) *reinterpret_cast<unsigned short*>(dst + d * stride) = digit62_bf16(v, d);
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
+    if (t == 0) {
+      tc_fence_after();
+      const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
+#pragma unroll 1
+      for (int slot = 0; slot < kEntS; slot++)
+#pragma unroll 1
+        for (int s = 0; s <= slot; s++)
+          mma_bf16<64>(tmem + slot * 64, smem_desc(a0 + s * kEntASlice), smem_desc(b0 + (slot - s) * kEntBSlice),
+                       s == 0 ? 0u : 1u);
+      mma_commit(&done);
+    }
+    load(u + gridDim.x);   // arrives beside the products and the stores
+    const bool ok = __syncthreads_and(mbar_wait(&done, phase, p.flag, p.wait_ns));
+    phase ^= 1;
+    if (!ok) break;   // the host sees the status bit
+    tc_fence_after();
+    const int row = (warp & 3) * 32 + lane, ea = eA[row];
+#pragma unroll 1
+    for (int part = 0; part < 2; part++) {
+      const int col0 = (warp >> 2) * 16 + part * 8;
+      if (col0 >= in) continue;
+      uint32_t r[kEntS][8];
+#pragma unroll
+      for (int s = 0; s < kEntS; s++)
+        tmem_ld8_async(tmem + ((uint32_t)((warp & 3) * 32) << 16) + s * 64 + col0, r[s]);
+      tmem_wait_ld();
+#pragma unroll
+      for (int s = 0; s < kEntS; s++) tmem_use8(r[s]);
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        int v[kEntS];
+#pragma unroll
+        for (int s = 0; s < kEntS; s++) v[s] = __float2int_rn(__uint_as_float(r[s][j]));
+        // sum_s v_s 256^(6 - s), the last level rounded in: below 2^63
+        const long long hi = v[0] * 65536 + v[1] * 256 + v[2];
+        const long long T = (hi << 32) + (long long)v[3] * 16777216 + (long long)v[4] * 65536 +
+                            (v[5] * 256 + v[6] + ((v[7] + 128) >> 8));
+        const int eb = eB[col0 + j];
+        out_tile[row * 65 + col0 + j] = (ea == kLayBad || eb == kLayBad) ? nan("") : scaled_int(T, ea + eb - 60);
+      }
+    }
+    tc_fence_before();
+    __syncthreads();
+    // coalesced: a warp stores one output's row of `in` columns at a time
+    for (int r = warp; r < 128; r += kLayThreads / 32) {
+      const int e = 2 * g + (r >> 6), o = r & 63;
+      const int64_t jr = p.row0 + (p.p0 + pl) * p.nr + e;
+      if (e >= p.nr || o >= out || jr < p.jlo || jr >= p.jhi) continue;
+      double* dst = p.J + (jr - p.jlo) * p.ldJ + p.net.offW[l] + (int64_t)o * in;
+      if (lane < in) dst[lane] = out_tile[r * 65 + lane];
+      if (lane + 32 < in) dst[lane + 32] = out_tile[r * 65 + lane + 32];
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(512));
   }
 }
 
@@ -796,7 +988,7 @@ int64_t lay_point_doubles(const NetDesc& net, int d, int nf, int ne, int mode) {
   int64_t n = 2 + nf * cf;
   for (int j = 1; j < net.L; j++) {
     if (j >= 2) n += (int64_t)cf * net.w[j];
-    if (mode != MODE_RESIDUAL) n += (int64_t)cr * net.w[j] * (1 + nr);
+    if (mode != MODE_RESIDUAL) n += (int64_t)cr * net.w[j] * (1 + nr) + (cr + 1) / 2;
   }
   if (mode != MODE_RESIDUAL) n += nr * nf * cr + 1 + 2 * (int64_t)nr * cr * kLayW;
   return n;
@@ -825,6 +1017,18 @@ cudaError_t run_gemm(const LayArgs& a, cudaStream_t st) {
   lay_gemm<D, C, KIND><<<(unsigned)grid, kLayThreads, kLaySmem, st>>>(a);
   count_launch();
   return cudaGetLastError();
+}
+
+// lay_hidden_entries always computes two rows by 64 outputs by 64 columns (and stops at the narrower
+// layer's columns); the FP64 form pays for what there is.  Jacobian, FP64 -> products, three hidden layers, 8192
+// points.  Two rows per point: width 40 1.96 -> 1.98 ms, 44 2.08 -> 2.04, 52 2.30 -> 2.11, 64 2.61 -> 2.20.
+// Three rows (every second pair half empty): 52 3.11 -> 3.19 ms, 56 3.27 -> 3.26, 60 3.45 -> 3.31,
+// 64 3.57 -> 3.31; 2048 points cross at the same widths.  A single row leaves half of every product empty.
+template <int D>
+bool hidden_entries(const NetDesc& net, int nr) {
+  bool wide = D == 2 && nr > 1;
+  for (int l = 1; l < net.L; l++) wide = wide && net.w[l] >= (nr % 2 ? 56 : 44);
+  return wide;
 }
 
 template <int EQ, int MODE>
@@ -857,8 +1061,10 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
     double* nn = take(NF * C);
     for (int j = 2; j < L; j++) Z[j] = take((int64_t)C * net.w[j]);
     double *seeds = nullptr, *lamg = nullptr;
+    int* He[GN_MAX_LAYERS + 1] = {};
     if (MODE != MODE_RESIDUAL) {
       for (int j = 1; j < L; j++) {
+        He[j] = reinterpret_cast<int*>(take((CR + 1) / 2));
         H[j] = take((int64_t)CR * net.w[j]);
         Ab[j] = take((int64_t)nr * CR * net.w[j]);
       }
@@ -902,6 +1108,7 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
       g.zin = Z[j];
       g.bias = A.theta + net.offB[j - 1];
       g.hout = H[j];
+      g.hexp = He[j];
       g.out = Z[j + 1];
       g.wsl = wsl + (size_t)(2 * (j - 1)) * opb;
       g.we = we + 2 * (j - 1) * kLayW;
@@ -964,6 +1171,10 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
     }
     en.seeds = seeds;
     en.J = A.J;
+    en.flag = A.flag + 2;
+    en.wait_ns = g.wait_ns;
+    en.hidden = !hidden_entries<D>(net, nr);
+    for (int j = 1; j < L; j++) en.He[j] = He[j];
     if (MODE == MODE_GRADIENT) {
       LayGrad gr = {en, lamg, parts, lay_ldg(net)};
       int tiles = 0, sums = net.w[1] * D + net.w[L] * net.w[L - 1] + 1;
@@ -980,6 +1191,14 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
     }
     lay_entries<D><<<(unsigned)((n * L + 7) / 8), 256, 0, st>>>(en);
     count_launch();
+    if (!en.hidden) {
+      if ((e = cudaFuncSetAttribute(lay_hidden_entries, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kEntSmem)) != cudaSuccess)
+        return e;
+      const int64_t units = n * (L - 2) * ((nr + 1) / 2);
+      lay_hidden_entries<<<(unsigned)(units < sm_count() ? units : sm_count()), kLayThreads, kEntSmem, st>>>(en);
+      count_launch();
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -34,7 +34,8 @@ def _rows(pick, ne):
 @pytest.mark.parametrize("name,hidden,n", [
     ("burgers", [24, 24], 4096), ("burgers", [32, 64, 33], 4111), ("ccf", [64, 64, 64], 4097), ("ccf", [31, 25], 4099),
     ("ipm", [64, 64, 64, 64], 2049), ("ipm", [40, 27, 64], 2200), ("boussinesq", [48, 48, 48], 2048),
-    ("boussinesq", [33, 64], 2061)])
+    ("boussinesq", [33, 64], 2061), ("boussinesq", [64, 56, 60], 2053), ("ipm", [44, 64], 2051),
+    ("ipm", [45, 44, 63], 2048)])
 def test_rows_and_jacobian_equal_the_pointwise_kernel(name, hidden, n):
     big, few, pick, pb, pf = _pair(name, hidden, n)
     ne = EQS[name][1]
@@ -125,6 +126,17 @@ def test_extreme_and_non_finite_values(name):
     assert pn.gn_residual(dev(big.theta), big.lam, r)[0] == -4
     bad = np.flatnonzero(~np.isfinite(host(r)))
     assert bad.size and set(bad) <= set(range(1234 * ne, 1234 * ne + ne))
+
+
+def test_jacobian_of_extreme_weights():
+    """Hidden weights' entries as products (2D, wide layers): components of very different sizes."""
+    big, few, pick, pb, pf = _pair("ipm", [48, 64, 48], 2100)
+    sel = torch.from_numpy(_rows(pick, 2)).cuda()
+    theta = big.theta.copy()
+    theta[::7] *= 40.0
+    theta[3::11] *= 1e-200
+    J_b, J_f = pb.jacobian(dev(theta), big.lam), pf.jacobian(dev(theta), big.lam)
+    assert rel(host(J_b[sel]), np.sqrt(len(pick) / 2100) * host(J_f[:2 * len(pick)])) <= TOL
 
 
 def test_step_graph_equals_step():
