@@ -736,9 +736,18 @@ def measured_peak(key, default):
         return default, "fallback"
 
 
-def gram_executed_flops(rows, Pp, S):
+def gram_by_residues(rows, Pp, S, args):
+    """The library's rule: six slices, no forced tile or split, at least P'/4 rows (ozaki.cu)."""
+    return S == 6 and not args.gram_split and not args.gram_tile and 4 * rows >= Pp
+
+
+def gram_executed_flops(rows, Pp, S, residues=False):
     """Tensor-pipe FLOP of one split Gram launch: S(S+1)/2 slice pairs over the 128 x 128
-    lower-triangular tiles of G and the 128-padded K (the Ozaki overhead included)."""
+    lower-triangular tiles of G and the 128-padded K (the Ozaki overhead included); or 13 residue
+    products over the 256 x 256 lower tiles and the 64-padded K."""
+    if residues:
+        nt = -(-Pp // 256)
+        return 13.0 * (nt * (nt + 1) / 2) * 256 * 256 * (-(-rows // 64) * 64) * 2.0
     nt = -(-Pp // 128)
     kpad = -(-rows // 128) * 128
     return S * (S + 1) / 2 * (nt * (nt + 1) / 2) * 128 * 128 * kpad * 2.0
@@ -749,8 +758,7 @@ def kernel_report(prob, args, phases, pipe_tiles=0):
 
     Gram: rows * P'(P'+1) FLOP (symmetric half).  FP64 path: DFMA pipe against the
     nominal FP64 peak.  Split paths: the tensor-pipe utilisation of the slice
-    products actually executed (S(S+1)/2 pairs over the 128 x 128 lower-triangular
-    tiles and the 128-padded K) against the measured sustained BF16 peak, plus the
+    products actually executed (gram_executed_flops) against the measured sustained BF16 peak, plus the
     FP64-equivalent TFLOP/s.  Cholesky: P'^3/3 FLOP; on the FP64 path against the
     DFMA pipe, on the SPLIT_ALL path reported as FP64-equivalent TFLOP/s only (its
     time is shared between the FP64 diagonal factors, which are latency-bound on one
@@ -770,24 +778,30 @@ def kernel_report(prob, args, phases, pipe_tiles=0):
     else:
         S = args.slices
         pk, src = measured_peak("bf16_tflops_sustained", 1700.0)
-        executed = gram_executed_flops(rows, Pp, S)
+        residues = gram_by_residues(rows, Pp, S, args)
+        executed = gram_executed_flops(rows, Pp, S, residues)
         tens = executed / (gram_ms * 1e-3) / 1e12
         alg = gram_flops / (gram_ms * 1e-3) / 1e12
         # DRAM bytes of the whole-triangle launch from one ncu capture; the pipelined step's
         # chunk launches run inside a graph with conditional nodes, where ncu lists no kernels
         traffic = (GRAM_TRAFFIC_BYTES_CCF_S6 if (S == 6 and getattr(args, "workload", "") == "ccf_unstable1"
-                                                 and not pipe_tiles) else None)
+                                                 and not pipe_tiles and not residues) else None)
         out["gram"] = {"bound": "tensor", "achieved": alg, "peak": pk, "unit": "TFLOP/s", "frac": alg / pk,
                        "achieved_units": "algorithmic FLOP rows * P'(P'+1) (the symmetric half of J~^T J~, "
                                          "FP64-equivalent) per launch / the Gram phase time; the split "
                                          "path's extra slice products count as overhead",
                        "tensor_pipe": {"executed_tflops": tens, "frac": tens / pk,
                                        "executed_flops_per_launch": executed,
-                                       "note": f"{S * (S + 1) // 2} BF16 slice-pair products per FP64-accurate "
+                                       "note": "13 BF16 residue products per FP64-accurate entry, over the 256 x 256 "
+                                               "lower tiles and 64-padded K" if residues else
+                                               f"{S * (S + 1) // 2} BF16 slice-pair products per FP64-accurate "
                                                "entry, over the 128 x 128 lower tiles and 128-padded K"},
                        "traffic": traffic, "traffic_unit": "bytes per launch" if traffic else None, "ms": gram_ms,
-                       "kernel": f"ozaki_kernel<{S},1,0> (split Gram: BF16 slice products on tcgen05, TMEM "
-                                 "accumulators; the slicing pre-pass is inside the timed phase)",
+                       "kernel": "crt_gemm (split Gram: exact BF16 residue products on tcgen05 CTA pairs, TMEM "
+                                 "accumulators; the residues and the reconstruction are inside the timed phase)"
+                       if residues else
+                       f"ozaki_kernel<{S},1,0> (split Gram: BF16 slice products on tcgen05, TMEM "
+                       "accumulators; the slicing pre-pass is inside the timed phase)",
                        "peak_source": src + ", sustained: the kernel runs inside a long step",
                        **({"pipelined": f"column-major chunks of <= {pipe_tiles} tiles on the lowest-priority "
                                         "stream beside the factorisation; ms is the Gram's wall time (slicing "
@@ -955,11 +969,13 @@ def batched_record(args, steps, warmup, rank=0, world=1):
         roof = None
         if prec != gn.GN_PREC_FP64:
             pk, src = measured_peak("bf16_tflops_sustained", 1700.0)
-            ex = sum(gram_executed_flops(r, p, args.slices) for r, p in zip(rows, Pps))
+            res = [gram_by_residues(r, p, args.slices, args) for r, p in zip(rows, Pps)]
+            ex = sum(gram_executed_flops(r, p, args.slices, q) for r, p, q in zip(rows, Pps, res))
             a = ex / (ms * 1e-3) / 1e12
             roof = {"bound": "tensor", "achieved": a, "peak": pk, "unit": "TFLOP/s", "frac": a / pk,
-                    "traffic": None, "kernel": f"ozaki_kernel<{args.slices},1> Gram launches of all fits",
-                    "note": "executed Gram slice-product FLOP of all fits / whole batched step time "
+                    "traffic": None, "kernel": ("crt_gemm" if all(res) else f"crt_gemm and ozaki_kernel<{args.slices},1>" if any(res)
+                               else f"ozaki_kernel<{args.slices},1>") + " Gram launches of all fits",
+                    "note": "executed Gram product FLOP of all fits / whole batched step time "
                             "(a lower bound on the Gram kernels' own rate)", "peak_source": src}
         line = {"metric": "gn_fit_steps_per_s", "value": value, "unit": "fit-steps/s", "n_gpus": world,
                 "steps": steps, "warmup": warmup, "ms_per_step": ms, "higher_is_better": True,

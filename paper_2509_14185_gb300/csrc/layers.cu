@@ -14,8 +14,8 @@
 //                 reverse-pass seeds (chain.cuh, the chain jet.cu evaluates per warp)
 //   lay_gemm      reverse, per hidden layer: abar_{j+1} = Hbar_{j+1} through the tanh jets,
 //                 Hbar_j = W_j^T abar_{j+1}
-//   lay_entries   the Jacobian rows sum_c abar_c[o] h_c[i]; or, for the gradient, their sums over the
-//                 points (lay_outer, lay_sums)
+//   lay_entries   the Jacobian rows sum_c abar_c[o] h_c[i] (lay_hidden_entries for wide 2D layers); or,
+//                 for the gradient, their sums over the points (lay_outer, lay_sums)
 //
 // Precision of the products: every row of either operand is scaled by a power of two and rounded to
 // a 55-bit integer (its largest element keeps two bits more than FP64's own 53), written as 7

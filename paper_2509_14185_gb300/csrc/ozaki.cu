@@ -1,7 +1,8 @@
 // Split-precision (Ozaki) GEMM on the tcgen05 tensor cores: C op= A B^T with
 // FP64 operands split into BF16 slices.  Used for the three dense
 // contractions of the Gauss-Newton step (Methods, "Second-order Optimizer"):
-// the Gram product G = J~^T J~, the CCF Hilbert contraction J_U = K J_g, and
+// the Gram product G = J~^T J~ (at six slices mostly by residues instead, crt.cu),
+// the CCF Hilbert contraction J_U = K J_g, and
 // the trailing updates of the blocked Cholesky factorisation.  GB300 runs
 // BF16 on its tensor cores ~1600x faster than FP64, so the FP64 values are
 // split and the slice products accumulated exactly (Ozaki, Ogita, Oishi &
