@@ -394,6 +394,8 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
                               (s == 0 && ks == 0 && kk == 0) ? 0u : 1u);
       mma_commit(&done);
     }
+    // (read here: behind the next barrier the producers of the next tile overwrite the exponents)
+    const int row = (warp & 3) * 32 + lane, ea = eA[row];
     ok = __syncthreads_and(mbar_wait(&done, phase, p.flag, p.wait_ns));
     phase ^= 1;
     if (!ok) {   // the host sees the status bit; this CTA's remaining rows become NaN
@@ -406,9 +408,8 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
     tc_fence_after();
     // ---- levels to FP64 ------------------------------------------------------------------------------
     {
-      const int row = (warp & 3) * 32 + lane, cg = warp >> 2;   // 16 columns per warp
+      const int cg = warp >> 2;   // 16 columns per warp
       const bool valid = row < ni * C;
-      const int ea = eA[row];
       const int64_t orow = i0 * C + row;
 #pragma unroll
       for (int part = 0; part < 2; part++) {

@@ -145,3 +145,27 @@ def test_step_graph_equals_step():
     ta, tb = dev(big.theta), dev(big.theta)
     a, b = pb.gn_step(ta, big.lam, 1e-2), pg.gn_step_graph(tb, big.lam, 1e-2)
     assert a[:3] == b[:3] and torch.equal(ta, tb)
+
+
+@pytest.mark.parametrize("name,hidden,n", [("burgers", [24, 24, 24], 300007), ("ipm", [32, 24, 30], 40001)])
+def test_tiles_keep_their_own_exponents(name, hidden, n):
+    """Many tiles per SM, outputs so narrow that half of the warps have no columns to combine, and
+    neighbouring tiles whose rows differ by orders of magnitude: a row scaled by another tile's
+    exponent would be off by a power of two."""
+    big, few, pick, _, _ = _pair(name, hidden, n)
+    # the near half of the points and the far half in turn, in stretches of one tile's points
+    order = np.argsort(np.abs(big.y).sum(0))
+    stretch = np.arange(n) // (64 if name == "burgers" else 21)
+    big.y[:] = big.y[:, order[np.argsort(stretch % 2, kind="stable").argsort()]]
+    few = dataclasses.replace(big, y=np.ascontiguousarray(big.y[:, pick]), rho=big.rho[pick])
+    pb, pf = gpu_problem(big), gpu_problem(few)
+    ne = EQS[name][1]
+    sel = torch.from_numpy(_rows(pick, ne)).cuda()
+    th = dev(big.theta)
+    m = len(pick) * ne
+    scale = np.sqrt(len(pick) / n)
+    ref = scale * host(pf.residual(th, big.lam)[0][:m])
+    first = pb.residual(th, big.lam)[0].clone()
+    assert rel(host(first[sel]), ref) <= TOL
+    for _ in range(5):
+        assert torch.equal(pb.residual(th, big.lam)[0], first)
