@@ -42,6 +42,8 @@ struct gn_batch {
   unsigned char* hs = nullptr;            // pinned host mirror
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
+  std::vector<double*> thetas;            // what the graph was captured with
+  std::vector<gn::GraphKey> keys;
 };
 
 namespace {
@@ -150,6 +152,9 @@ int gn_batch_capture_graph(gn_batch* b, double* const* thetas) {
     return rc != GN_OK ? rc : GN_ERR_CUDA;
   }
   b->graph = g;
+  b->thetas.assign(thetas, thetas + b->n_fits);
+  b->keys.clear();
+  for (gn_handle* h : b->handles) b->keys.emplace_back(h);
   if (GN_NOTE(cudaGraphInstantiate(&b->exec, g, cudaGraphInstantiateFlagUseNodePriority)) != cudaSuccess) {
     release_graph(b);
     return GN_ERR_CUDA;
@@ -160,6 +165,22 @@ int gn_batch_capture_graph(gn_batch* b, double* const* thetas) {
 int gn_batch_graph_step(gn_batch* b, double* lambdas, double* dampings, gn_step_info* infos, int* status) {
   if (!b || !lambdas || !dampings) return GN_ERR_INVALID;
   if (!b->exec) return GN_ERR_INVALID;   // gn_batch_capture_graph first
+  // A call on one of the fits' handles may have moved a workspace whose address the graph holds:
+  // capture again, with the settings of the first capture.
+  bool moved = false;
+  for (int f = 0; f < b->n_fits; f++) moved = moved || b->handles[f]->ws_moves != b->keys[f].ws_moves;
+  if (moved) {
+    const std::vector<double*> thetas = b->thetas;
+    const std::vector<gn::GraphKey> keys = b->keys;
+    std::vector<gn::GraphKey> now;
+    for (int f = 0; f < b->n_fits; f++) {
+      now.emplace_back(b->handles[f]);
+      keys[f].apply(b->handles[f]);
+    }
+    const int rc = gn_batch_capture_graph(b, thetas.data());
+    for (int f = 0; f < b->n_fits; f++) now[f].apply(b->handles[f]);
+    if (rc) return rc;
+  }
   const size_t sb = gn::graph_state_bytes();
   for (int f = 0; f < b->n_fits; f++) gn::graph_host_state(b->handles[f], lambdas[f], dampings[f], b->hs + sb * f);
   if (GN_NOTE(cudaMemcpyAsync(b->ds, b->hs, sb * b->n_fits, cudaMemcpyHostToDevice, b->origin)) != cudaSuccess ||

@@ -1241,6 +1241,7 @@ int ensure_chol_ws(gn_handle* h, size_t need) {
     return GN_ERR_UNSUPPORTED;
   }
   if (h->chol_ws) cudaFree(h->chol_ws);   // synchronises: no kernel still reads it
+  h->ws_moves++;   // (graphs captured with the old one are stale)
   h->chol_ws = nullptr;
   h->chol_ws_bytes = 0;
   if (GN_NOTE(cudaMalloc(&h->chol_ws, need)) != cudaSuccess) return GN_ERR_OOM;

@@ -163,6 +163,8 @@ struct gn_handle {
   // split_ws so that it can run while the Gram still reads its operand
   void* chol_ws = nullptr;
   size_t chol_ws_bytes = 0;
+  // counts the (re)allocations of split_ws and chol_ws: a captured graph holds their addresses
+  int64_t ws_moves = 0;
   // pipelined step: the Gram runs as column-major chunks of at most pipe_tiles 128 x 128 tiles
   // beside the factorisation (0, the default: off, Gram then factorisation; -1: chosen from
   // the SM count)
@@ -216,6 +218,32 @@ int gram_into(gn_handle* h, const double* J, int64_t ld, int64_t nrows, const do
 // grow the split workspace to what every split contraction of a step needs, and create the
 // factorisation's streams, so that a captured step allocates nothing
 int prepare_for_capture(gn_handle* h);
+// What a captured step is built from beside theta: the handle's settings, and the addresses of its
+// workspaces (by the count of their moves).  A graph whose key differs from the handle's is stale.
+struct GraphKey {
+  int precision, n_slices, lam_frozen, staged, pipe_tiles, gram_ksplit, gram_tile, crt_off;
+  double stage_eps;
+  int64_t ws_moves;
+  explicit GraphKey(const gn_handle* h)
+      : precision(h->precision), n_slices(h->n_slices), lam_frozen(h->lam_frozen), staged(h->staged),
+        pipe_tiles(h->pipe_tiles), gram_ksplit(h->gram_ksplit), gram_tile(h->gram_tile), crt_off(h->crt_off),
+        stage_eps(h->stage_eps), ws_moves(h->ws_moves) {}
+  bool operator==(const GraphKey& o) const {
+    return precision == o.precision && n_slices == o.n_slices && lam_frozen == o.lam_frozen && staged == o.staged &&
+           pipe_tiles == o.pipe_tiles && gram_ksplit == o.gram_ksplit && gram_tile == o.gram_tile &&
+           crt_off == o.crt_off && stage_eps == o.stage_eps && ws_moves == o.ws_moves;
+  }
+  void apply(gn_handle* h) const {   // the settings, not the workspaces
+    h->precision = precision;
+    h->n_slices = n_slices;
+    h->lam_frozen = lam_frozen;
+    h->staged = staged;
+    h->pipe_tiles = pipe_tiles;
+    h->gram_ksplit = gram_ksplit;
+    h->gram_tile = gram_tile;
+    h->stage_eps = stage_eps;
+  }
+};
 size_t chol_split_ws_bytes(int64_t n, int S);
 // split-K factor and tile width the Gram autotuner recorded for this shape (0: not tuned yet)
 int gram_split_choice(int S, int64_t Pp, int64_t nrows);

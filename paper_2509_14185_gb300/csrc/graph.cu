@@ -69,11 +69,11 @@ struct GraphState {
   // 6 model scalars done, 7 commit done; 3 is unused
   cudaEvent_t evp[8] = {};
   bool marks = false;   // the graphs carry the marks (one row block; not a batch branch)
-  int precision = -1, n_slices = -1, lam_frozen = -1, staged = -1, pipe = -2;   // of the handle when captured
-  double stage_eps = 0.0;
+  GraphKey key;         // of the handle when captured
   // kernels per replay, for gn_kernel_launches: outside the trial bodies (step graph, solve
   // graph, a batch's step branch) and per line-search trial that runs
   long long k_step = 0, k_solve = 0, k_branch = 0, k_trial = 0;
+  explicit GraphState(const gn_handle* h) : key(h) {}
 };
 
 namespace {
@@ -369,7 +369,7 @@ void destroy_graphs(GraphState* gs) {
 // Per-handle graph state (device state, pinned mirror, streams, timing events).
 int ensure_state(gn_handle* h, StepState* external_ds) {
   if (!h->gs) {
-    GraphState* gs = new (std::nothrow) GraphState;
+    GraphState* gs = new (std::nothrow) GraphState(h);
     if (!gs) return GN_ERR_OOM;
     h->gs = gs;
     if (GN_NOTE(cudaMallocHost((void**)&gs->hs, sizeof(StepState))) != cudaSuccess) return GN_ERR_OOM;
@@ -418,12 +418,7 @@ int build_graphs(gn_handle* h, double* theta, bool with_step) {
   if (with_step) GN_G_TRY(cudaGraphInstantiate(&gs->x_step, gs->g_step, cudaGraphInstantiateFlagUseNodePriority));
   GN_G_TRY(cudaGraphInstantiate(&gs->x_solve, gs->g_solve, cudaGraphInstantiateFlagUseNodePriority));
   gs->theta = theta;
-  gs->precision = h->precision;
-  gs->n_slices = h->n_slices;
-  gs->lam_frozen = h->lam_frozen;
-  gs->staged = h->staged;
-  gs->stage_eps = h->stage_eps;
-  gs->pipe = h->pipe_tiles;
+  gs->key = GraphKey(h);
   return GN_OK;
 }
 
@@ -538,9 +533,7 @@ int gn_step_graph(gn_handle* h, double* theta, double* lambda, double* damping, 
   int rc = ensure_state(h, nullptr);
   if (rc) return rc;
   GraphState* gs = h->gs;
-  if (gs->theta != theta || !gs->x_step || gs->precision != h->precision || gs->n_slices != h->n_slices ||
-      gs->lam_frozen != h->lam_frozen || gs->staged != h->staged || gs->stage_eps != h->stage_eps ||
-      gs->pipe != h->pipe_tiles) {
+  if (gs->theta != theta || !gs->x_step || !(gs->key == GraphKey(h))) {
     rc = build_graphs(h, theta, true);
     if (rc) return rc;
   }

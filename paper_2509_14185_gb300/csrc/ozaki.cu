@@ -917,6 +917,7 @@ int ensure_split_ws(gn_handle* h, size_t need) {
     return GN_ERR_UNSUPPORTED;
   }
   if (h->split_ws) cudaFree(h->split_ws);   // synchronises: no kernel still reads it
+  h->ws_moves++;   // (graphs captured with the old one are stale)
   h->split_ws = nullptr;
   h->split_ws_bytes = 0;
   if (GN_NOTE(cudaMalloc(&h->split_ws, need)) != cudaSuccess) return GN_ERR_OOM;
