@@ -534,7 +534,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 
 // Sizes of a residue Gram of n columns: how many of nrows rows go into one product (the planes stay
 // within what the six slices of ozaki.cu would take, or 6 GB), the tiles whose residues are kept at once, and
-// the bytes of all that.
+// the bytes of all that.  The bytes never fall as nrows grows, so a workspace for the largest row block serves
+// the shorter ones.
 CrtPlan crt_plan(int64_t n, int64_t nrows) {
   CrtPlan pl;
   pl.npad = rup(n > 0 ? n : 1, CT);
@@ -544,8 +545,8 @@ CrtPlan crt_plan(int64_t n, int64_t nrows) {
   int64_t k = cap / (NP * pl.npad * 2) / KS * KS;
   if (k < KS) k = KS;
   if (k > kMaxRows) k = kMaxRows;
-  const int64_t blocks = (all + k - 1) / k;
-  pl.krows = rup((all + blocks - 1) / blocks, KS);
+  // the last product takes what is left: products of equal size would need less memory for slightly more rows
+  pl.krows = k < all ? k : all;
   const int64_t mt = pl.npad / CT, tiles = mt * (mt + 1) / 2;
   pl.batch = tiles < 8 * 76 ? tiles : 8 * 76;
   pl.planes = rup(NP * pl.npad * pl.krows * 2, 1024);

@@ -1078,13 +1078,22 @@ void record_default_choice(const gn_handle* h, int64_t nrows) {
   std::lock_guard<std::mutex> g(g_tune_mu);
   g_tune.emplace(std::make_tuple(h->n_slices, (h->Pp + TM - 1) / TM, gram_chunks(nrows)), GramChoice());
 }
-// false: no memory for the planes (remembered), the slices have to do
-bool residue_ws(gn_handle* h, int64_t nrows) {
-  if (!by_residues(h, nrows)) return false;
-  if (ensure_split_ws(h, residue_bytes(h, nrows)) == GN_OK) return true;
+// Does a Gram of nrows rows go by residues?  No memory for the planes is remembered (the slices have
+// to do from then on); any other failure is the caller's.
+int residue_ws(gn_handle* h, int64_t nrows, bool* yes) {
+  *yes = false;
+  if (!by_residues(h, nrows)) return GN_OK;
+  const int rc = ensure_split_ws(h, residue_bytes(h, nrows));
+  *yes = rc == GN_OK;
+  if (rc != GN_ERR_OOM) return rc;
   cudaGetLastError();
   h->crt_off = 1;
-  return false;
+  return GN_OK;
+}
+// the bytes of a Gram of nrows rows by slices
+size_t slice_bytes(gn_handle* h, int64_t nrows) {
+  return oz_operand_bytes(h->n_slices, h->Pp, nrows) + colmax_bytes(h->Pp) +
+         gram_part_bytes(h->Pp, gram_max_split(h, nrows));
 }
 }  // namespace
 
@@ -1115,8 +1124,15 @@ int prepare_for_capture(gn_handle* h) {
   if (GN_NOTE(ensure_chol_streams(h)) != cudaSuccess) return GN_ERR_CUDA;
   if (h->precision == GN_PREC_FP64) return GN_OK;
   const int S = h->n_slices;
-  size_t need = oz_operand_bytes(S, h->Pp, h->jrows) + (size_t)CM_CHUNKS * rup(h->Pp, TM) * 8 + 256 +
-                gram_part_bytes(h->Pp, gram_max_split(h, h->jrows));
+  // the row blocks of a step: jrows rows and the remainder (which may take more split-K parts)
+  const int64_t blocks[2] = {h->jrows, h->jrows > 0 ? h->n_rows % h->jrows : 0};
+  size_t need = 0, planes = 0;
+  for (int64_t rows : blocks) {
+    if (rows <= 0) continue;
+    const size_t s = slice_bytes(h, rows), p = by_residues(h, rows) ? residue_bytes(h, rows) : 0;
+    need = s > need ? s : need;
+    planes = p > planes ? p : planes;
+  }
   if (h->precision == GN_PREC_SPLIT_ALL) {
     if (h->eq == GN_CCF && h->p.n_pts > 0) {
       const int64_t rows = h->p.n_pts < h->jrows ? h->p.n_pts : h->jrows;
@@ -1127,9 +1143,9 @@ int prepare_for_capture(gn_handle* h) {
     const int rc = ensure_chol_ws(h, chol_split_ws_bytes(h->Pp, S));
     if (rc) return rc;
   }
-  if (by_residues(h, h->jrows)) {   // the planes when they can be had, else the slices
-    const size_t planes = residue_bytes(h, h->jrows);
-    if (ensure_split_ws(h, planes > need ? planes : need) == GN_OK) return pretune_gram(h);
+  if (planes > 0) {   // the planes when they can be had, else the slices
+    const int rc = ensure_split_ws(h, planes > need ? planes : need);
+    if (rc != GN_ERR_OOM) return rc ? rc : pretune_gram(h);
     cudaGetLastError();
     h->crt_off = 1;
   }
@@ -1143,12 +1159,15 @@ int split_gram(gn_handle* h, const double* J, int64_t ld, int64_t nrows, double*
   const int S = h->n_slices;
   if (S < 1 || S > kOzMaxSlices) return GN_ERR_UNSUPPORTED;
   if (nrows <= 0) return GN_OK;
-  if (residue_ws(h, nrows)) {
+  bool residues;
+  int rc = residue_ws(h, nrows, &residues);
+  if (rc) return rc;
+  if (residues) {
     const CrtPlan pl = crt_plan(h->Pp, nrows);
     double* part = reinterpret_cast<double*>(static_cast<unsigned char*>(h->split_ws) + pl.bytes);
     for (int64_t k0 = 0; k0 < nrows; k0 += pl.krows) {
       const int64_t k = k0 + pl.krows < nrows ? pl.krows : nrows - k0;
-      int rc = crt_prepare(pl, J + k0 * ld, ld, k, h->Pp, h->split_ws, part, h->st);
+      rc = crt_prepare(pl, J + k0 * ld, ld, k, h->Pp, h->split_ws, part, h->st);
       if (!rc)
         rc = crt_product(pl, k, h->Pp, h->split_ws, G, h->Pp, accumulate || k0 > 0, 0, -1, 0, 0, h->flag + 2, h->st);
       if (rc) return rc;
@@ -1158,7 +1177,7 @@ int split_gram(gn_handle* h, const double* J, int64_t ld, int64_t nrows, double*
   }
   const size_t opb = oz_operand_bytes(S, h->Pp, nrows);
   const size_t cmb = colmax_bytes(h->Pp);
-  int rc = ensure_split_ws(h, opb + cmb + gram_part_bytes(h->Pp, gram_max_split(h, nrows)));
+  rc = ensure_split_ws(h, slice_bytes(h, nrows));
   if (rc) return rc;
   OzOperand op = oz_operand_at(h->split_ws, S, h->Pp, nrows);
   double* part = reinterpret_cast<double*>(static_cast<unsigned char*>(h->split_ws) + opb);
@@ -1206,17 +1225,17 @@ int split_gram_pipelined(gn_handle* h, const double* J, int64_t ld, int64_t nrow
   const int S = h->n_slices;
   const int64_t n = h->Pp;
   if (S < 1 || S > kOzMaxSlices || nrows <= 0 || chunk <= 0) return GN_ERR_INVALID;
-  const bool residues = residue_ws(h, nrows);
+  bool residues;
+  int rc = residue_ws(h, nrows, &residues);
+  if (rc) return rc;
   const CrtPlan pl = crt_plan(n, nrows);
   const size_t opb = oz_operand_bytes(S, n, nrows);
-  const size_t cmb = colmax_bytes(n);
   OzOperand op;
-  int rc = GN_OK;
   if (residues) {
     rc = crt_prepare(pl, J, ld, nrows, n, h->split_ws,
                      reinterpret_cast<double*>(static_cast<unsigned char*>(h->split_ws) + pl.bytes), st);
   } else {
-    rc = ensure_split_ws(h, opb + cmb + gram_part_bytes(n, gram_max_split(h, nrows)));
+    rc = ensure_split_ws(h, slice_bytes(h, nrows));
     if (rc) return rc;
     op = oz_operand_at(h->split_ws, S, n, nrows);
     rc = oz_prepare_cols(S, J, ld, nrows, n, op,

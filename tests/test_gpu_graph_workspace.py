@@ -70,3 +70,32 @@ def test_batch_graph_after_a_moved_workspace():
         assert (le, ge, se) == (lg, gg, sg)
         assert all(torch.equal(x, y) for x, y in zip(te, tg))
     assert all(np.all(np.isfinite(host(t))) for t in tg)
+
+
+@pytest.mark.parametrize("precision", [1, 2])
+def test_streamed_step_with_a_remainder(precision):
+    """Row blocks of more rows than one product of residues takes, the last block shorter: the captured
+    step equals the eager one, the Gram stays on the residues, and no row count up to the
+    block's needs more memory than the step."""
+    w = I.small_case(I.BURGERS, [1, 20, 20, 1], 63000)
+    pe = gpu_problem(w, precision=precision, n_slices=6, row_block=33000)
+    pg = gpu_problem(w, precision=precision, n_slices=6, row_block=33000)
+    te, tg = dev(w.theta), dev(w.theta)
+    a, b = pe.gn_step(te, w.lam, 1e-2), pg.gn_step_graph(tg, w.lam, 1e-2)
+    assert a[:3] == b[:3] and torch.equal(te, tg)
+    n = pg.P + 1
+    J = torch.randn(33000, n, dtype=torch.float64, device="cuda")
+    ref = torch.tril(J[:31000].T @ J[:31000])
+    G = torch.zeros(n, n, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    for rows in (32768, 30001, 16512, 1000, 33000, 31000):
+        pg.gn_gram(J, rows, None, G, None, precision=1)
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] == free
+    # slices would be off by their FP32 sums, near 1e-10
+    assert float((torch.tril(G) - ref).abs().max() / ref.abs().max()) <= 1e-13
+    a, b = pe.gn_step(te, a[1], a[2]), pg.gn_step_graph(tg, b[1], b[2])
+    assert a[:3] == b[:3] and torch.equal(te, tg)
+    pe.close()
+    pg.close()
