@@ -17,12 +17,18 @@
 //   lay_entries   the Jacobian rows sum_c abar_c[o] h_c[i] (lay_hidden_entries for wide 2D layers); or,
 //                 for the gradient, their sums over the points (lay_outer, lay_sums)
 //
-// Precision of the products: every row of either operand is scaled by a power of two and rounded to
-// a 55-bit integer (its largest element keeps two bits more than FP64's own 53), written as 7
-// balanced base-256 digits (exact in BF16).  The 28 digit pairs of the seven leading levels are summed
-// per level in FP32 accumulators, exactly (at most 7 * 64 products below 2^14 each: < 2^23), and the levels are
-// combined in 64-bit integers and rounded once.  What is dropped lies 2^-55 below the largest products, under
-// the rounding of an FP64 sum of 64 terms.
+// Precision of the products: that of an FP64 sum, for every element.  A power of two per contraction index
+// (2^c_k, from the weights alone) moves from the weights to the activations, which evens out neurons of
+// different scale; then every row of either operand is scaled by a power of two 2^-e and rounded to a 62-bit
+// integer, written as 8 balanced base-256 digits, digit q in units of 256^-q (exact in BF16).  The digit pairs of
+// the eight leading levels are summed in FP32 accumulators: levels 0 to 5 each in its own, exactly (at most 6 * 64
+// products of at most 2^14 units), levels 6 and 7 in one; one more takes S, the sum of the products' magnitudes, from
+// BF16 forms of the operands rounded down.  The levels are combined in 64-bit integers and rounded once.
+// In units of 2^(e_a + e_w) an element of n terms is off by at most n 7.03 2^-62 for the missing levels (7 pairs of digits
+// of at most 2^7 on the first of them, 2^64 * 2^12 below the unit), n 2^-62 for the operands' roundings and 2.8 n 2^-60 for
+// the 15 ceil(n / 16) additions of the last accumulator, each off by at most two of its units of 2^-60: less than n 2^-57.7
+// together.  The FP64 sum is off by up to n 2^-53 S; so wherever S >= 2^-4.7 2^(e_a + e_w) the element is as good, and
+// elsewhere, or with an operand that is not finite, it is summed in FP64 (lay_exact; no element of a Xavier network).
 #include <cmath>
 #include <cstring>
 
@@ -32,14 +38,16 @@
 namespace gn {
 namespace {
 
-constexpr int kLayS = 7;                           // digits per value
+constexpr int kLayS = 8;                           // digits per value
+constexpr int kLaySl = kLayS + 1;                  // slices of an operand: the digits and the magnitude
 constexpr int kLayW = 64;                          // widest hidden layer
 constexpr int kLayThreads = 512;
-constexpr int kLayASlice = 2 * 128 * 64;           // one digit of the A tile: two 32-wide K stages
-constexpr int kLayWSlice = 2 * kLayW * 64;         // one digit of the weights
-constexpr int kLayA = kLayS * kLayASlice;          // 112 KB
-constexpr size_t kLaySmem = 1024 + kLayA + kLayS * kLayWSlice + 1024;
+constexpr int kLayASlice = 2 * 128 * 64;           // one slice of the A tile: two 32-wide K stages
+constexpr int kLayWSlice = 2 * kLayW * 64;         // one slice of the weights
+constexpr int kLayA = kLaySl * kLayASlice;         // 144 KB
+constexpr size_t kLaySmem = 1024 + kLayA + kLaySl * kLayWSlice + 1024;
 constexpr int kLayBad = 0x3fffffff;                // exponent of a row with a non-finite element
+constexpr int kLayZero = -100000;                  // exponent of a row of zeros
 
 struct LayArgs {
   int64_t items;            // points (forward) or points x rows (reverse)
@@ -59,8 +67,11 @@ struct LayArgs {
   const double* hbar;       // reverse: [item][CR][K]
   double* abar;             // reverse out: [item][CR][K]
   double* out;              // [item][C][N]
-  const unsigned char* wsl; // weight digits, kLayS x 64 x 64 BF16
+  const unsigned char* wsl; // weight slices, kLaySl x 64 x 64 BF16
   const int* we;            // weight exponents [64]
+  const int* wc;            // powers c_k of the contraction's indices [64]
+  const double* W;          // the weights themselves: element (output o, index k) at W[o * wso + k * wsk]
+  int64_t wso, wsk;
   int* flag;
   unsigned long long wait_ns;
 };
@@ -139,41 +150,49 @@ __device__ __forceinline__ void first_layer(const double* W0, const double* b0, 
 __device__ __forceinline__ unsigned abs_hi(double x) {
   return (unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu;
 }
-// e with 2^e > every |x| whose largest high word is m (kLayBad: one of them is not finite)
-__device__ __forceinline__ int row_exponent(unsigned m) {
-  const int ex = (int)(m >> 20);
-  return ex == 0x7ff ? kLayBad : (ex > 0 ? ex : 1) - 1022;
+// e with 2^e > |x| 2^c (kLayZero: x = 0, kLayBad: x is not finite); a row's exponent is the largest
+__device__ __forceinline__ int exponent_above(double x, int c) {
+  const int ex = (int)(abs_hi(x) >> 20);
+  int e = ex - 1022 + c;
+  if ((unsigned)(ex - 1) >= 0x7feu)   // rare: one branch for the normal numbers
+    e = ex ? kLayBad : (unsigned long long)__double_as_longlong(x) << 1 ? 1 - 1022 + c : kLayZero;
+  return e;
 }
-// x 2^(55 - e) to the nearest integer plus the digits' bias: bytes 0..5 are then digits 6..1 plus
-// 128 and the rest, shifted right arithmetically, is digit 0.
-__device__ __forceinline__ long long biased_digits(double x, int e) {
+// x 2^(62 - e) to the nearest integer plus the digits' bias (|x| <= 2^e; far above |x|: 0): byte 7 - q is
+// then digit q plus 128, |digit 0| <= 64
+constexpr unsigned long long kDigitBias = 0x8080808080808080ull;
+__device__ __forceinline__ unsigned long long biased_digits(double x, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7ff);
   unsigned long long m = b & 0xFFFFFFFFFFFFFull;
   if (ex > 0) m |= 1ull << 52;
-  const int sh = (ex > 0 ? ex : 1) - 1020 - e;   // <= 2
+  const int sh = (ex > 0 ? ex : 1) - 1013 - e;   // <= 9
   unsigned long long v;
-  if (sh >= 0) v = m << sh;
+  if (sh >= 0) v = sh > 9 ? 0ull : m << sh;
   else v = sh < -54 ? 0ull : (m + (1ull << (-sh - 1))) >> -sh;
-  return ((b >> 63) ? -(long long)v : (long long)v) + 0x808080808080ll;
+  return ((b >> 63) ? 0ull - v : v) + kDigitBias;
 }
-// digit q of a biased value as BF16 bits (an integer of at most 8 significant bits: the upper half
-// of its FP32 form)
-__device__ __forceinline__ unsigned short digit_bf16(long long u, int q) {
-  const unsigned lo = (unsigned)u, hi = (unsigned)((unsigned long long)u >> 32);
-  float f;
-  if (q == 0) f = (float)((int)hi >> 16);
-  else {
-    const int byte = 6 - q;   // 0..5
-    f = __uint_as_float(__byte_perm(byte < 4 ? lo : hi, 0x4B000000u, 0x7540 + (byte & 3))) - 8388736.0f;
-  }
+// digit q of a biased value, times 256^-q, as BF16 bits (at most 8 significant bits: the upper half of its
+// FP32 form).  The byte goes to the low end of the significand of 2^(23 - 8 q).
+__device__ __forceinline__ unsigned short digit_bf16(unsigned long long u, int q) {
+  const int byte = 7 - q;
+  const unsigned w = byte < 4 ? (unsigned)u : (unsigned)(u >> 32), base = 0x4B000000u - ((unsigned)q << 26);
+  const float f = __uint_as_float(__byte_perm(w, base, 0x7640 + (byte & 3))) - __uint_as_float(base | 128u);
   return (unsigned short)(__float_as_uint(f) >> 16);
 }
+// |x| 2^-e < 1 as BF16 bits, rounded down (0 below 2^-126)
+__device__ __forceinline__ unsigned short magnitude_bf16(double x, int e) {
+  const unsigned h = abs_hi(x);
+  const int ex = (int)(h >> 20) - 896 - e;
+  return ex > 0 && ex < 128 ? (unsigned short)(ex << 7 | (h >> 13 & 0x7f)) : (unsigned short)0;
+}
+constexpr int kNoDigits = 5000;   // an exponent far above every value: all slices zero
 // byte offset of element (row, k) in a K-major operand tile with the 64-byte swizzle, `rows` rows
 __device__ __forceinline__ int swz(int row, int k, int rows) {
   return (k >> 5) * rows * 64 + row * 64 + ((((k & 31) >> 3) ^ ((row >> 1) & 3)) << 4) + (k & 7) * 2;
 }
 
+__device__ __noinline__ double scaled_int_edge(long long T, int k) { return ldexp((double)T, k); }
 // T 2^k rounded to nearest even, by integer operations (an I2F and a multiply would take two slots of the FP64
 // pipe per element); FP64 where the result leaves the normal range
 __device__ __forceinline__ double scaled_int(long long T, int k) {
@@ -181,7 +200,7 @@ __device__ __forceinline__ double scaled_int(long long T, int k) {
   const unsigned long long m = T < 0 ? (unsigned long long)-T : (unsigned long long)T;
   const int lz = __clzll((long long)m);
   const int e = 1023 + 63 - lz + k;
-  if (e <= 0 || e >= 2046) return ldexp((double)T, k);
+  if (e <= 0 || e >= 2046) return scaled_int_edge(T, k);   // (a call: as a predicated instruction it costs its slot)
   const unsigned long long n = m << lz;                       // leading one at bit 63
   const unsigned long long rem = n & 0x7ff;
   unsigned long long r = ((unsigned long long)(e - 1) << 52) + (n >> 11);   // the leading one carries into e
@@ -198,8 +217,9 @@ struct LayPrep {
   double* qb;
   const double* theta;
   NetDesc net;
-  unsigned char* wsl;       // [(layer - 1) * 2 + direction][kLayS][64][64] BF16
+  unsigned char* wsl;       // [(layer - 1) * 2 + direction][kLaySl][64][64] BF16
   int* we;                  // [...][64]
+  int* wc;                  // [...][64]
   int pt_blocks;
 };
 template <int D>
@@ -220,47 +240,146 @@ __global__ void __launch_bounds__(256) lay_inputs(const LayPrep p) {
     p.qb[2 * i + 1] = D == 2 ? y1 / sqrt(u) : 0.0;
     return;
   }
-  // weights: one warp per operand row.  Forward operand of layer l: row o is W_l[o][.]; reverse:
-  // row i is W_l[.][i].
-  const int w = ((int)blockIdx.x - p.pt_blocks) * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int op = w / kLayW, row = w % kLayW, l = 1 + op / 2, rev = op & 1;
-  if (l > p.net.L - 2) return;
+  // weights, one warp per operand row, 8 rows per block.  Forward operand of layer l: row o is
+  // W_l[o][.]; reverse: row i is W_l[.][i].
+  const int t = threadIdx.x, wb = (int)blockIdx.x - p.pt_blocks, lane = t & 31;
+  const int op = wb / (kLayW / 8), row = wb % (kLayW / 8) * 8 + (t >> 5), l = 1 + op / 2, rev = op & 1;
   const int in = p.net.w[l], out = p.net.w[l + 1];
+  const int nrow = rev ? in : out, nk = rev ? out : in;
   const double* W = p.theta + p.net.offW[l];
+  auto weight = [&](int r, int k) {
+    const int o = rev ? k : r, i = rev ? r : k;
+    return (r < nrow && k < nk) ? W[(int64_t)o * in + i] : 0.0;
+  };
+  // The contraction index k's power c_k: the mean exponent of its weights.  Weights 2^16 and more below
+  // the largest count as 2^-16 of it, so that zeros and outliers hardly move it; a column times a
+  // power of two moves by exactly that.
+  __shared__ int top[4][kLayW], sum[4][kLayW], cnt[4][kLayW], cs[kLayW];
+  {
+    const int k = t & 63, g = t >> 6;
+    int ex[kLayW / 4], m = kLayZero;
+#pragma unroll
+    for (int q = 0; q < kLayW / 4; q++) {
+      const int r = g + 4 * q;
+      const int e = exponent_above(weight(r, k), 0);
+      ex[q] = r >= nrow || e == kLayBad ? kLayBad : e;   // (not counted)
+      if (ex[q] != kLayBad) m = ex[q] > m ? ex[q] : m;
+    }
+    top[g][k] = m;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; q++) m = top[q][k] > m ? top[q][k] : m;
+    int s = 0, n = 0;
+#pragma unroll
+    for (int q = 0; q < kLayW / 4; q++)
+      if (ex[q] != kLayBad) {
+        s += ex[q] > m - 16 ? ex[q] : m - 16;
+        n++;
+      }
+    sum[g][k] = s;
+    cnt[g][k] = n;
+    __syncthreads();
+    if (t < kLayW) {
+      s = sum[0][k] + sum[1][k] + sum[2][k] + sum[3][k];
+      n = cnt[0][k] + cnt[1][k] + cnt[2][k] + cnt[3][k];
+      cs[k] = m == kLayZero ? 0 : (int)floorf((float)s / (float)n + 0.5f);
+      if (row == t >> 5) p.wc[op * kLayW + k] = cs[k];   // (the first of the operand's blocks)
+    }
+    __syncthreads();
+  }
   double x[2];
-  unsigned m = 0;
+  int e = kLayZero;
 #pragma unroll
   for (int q = 0; q < 2; q++) {
     const int k = lane + 32 * q;
-    const int o = rev ? k : row, i = rev ? row : k;
-    x[q] = (o < out && i < in) ? W[(int64_t)o * in + i] : 0.0;
-    const unsigned h = abs_hi(x[q]);
-    m = h > m ? h : m;
+    x[q] = weight(row, k);
+    const int ek = exponent_above(x[q], -cs[k]);
+    e = ek > e ? ek : e;
   }
-  m = __reduce_max_sync(0xffffffffu, m);
-  const int e = row_exponent(m);
+  e = __reduce_max_sync(0xffffffffu, e);
   if (lane == 0) p.we[op * kLayW + row] = e;
-  unsigned short* dst = reinterpret_cast<unsigned short*>(p.wsl) + (size_t)op * kLayS * kLayW * kLayW + row * kLayW;
+  unsigned short* dst = reinterpret_cast<unsigned short*>(p.wsl) + (size_t)op * kLaySl * kLayW * kLayW + row * kLayW;
 #pragma unroll
   for (int q = 0; q < 2; q++) {
-    const long long u = biased_digits(x[q], e == kLayBad ? 0 : e);
+    const int k = lane + 32 * q, ek = e == kLayBad || e == kLayZero ? kNoDigits : e + cs[k];
+    const unsigned long long u = biased_digits(x[q], ek);
 #pragma unroll
-    for (int s = 0; s < kLayS; s++) dst[s * kLayW * kLayW + lane + 32 * q] = digit_bf16(u, s);
+    for (int s = 0; s < kLayS; s++) dst[s * kLayW * kLayW + k] = digit_bf16(u, s);
+    dst[kLayS * kLayW * kLayW + k] = magnitude_bf16(x[q], ek);
   }
 }
 
 // ---- one hidden layer ------------------------------------------------------------------------------
 enum LayKind : int { LAY_FWD_FIRST = 0, LAY_FWD = 1, LAY_REV_LAST = 2, LAY_REV = 3 };
 
+// the operand's elements at index k of an item: FP64 jets through tanh, or the adjoint through them
+template <int D, int C, int KIND>
+__device__ __forceinline__ void lay_operand(const LayArgs& p, int64_t item, int64_t pt, int k, double q, double beta,
+                                            double* x) {
+  constexpr int CR = JT<D>::CR;
+  if constexpr (KIND <= LAY_FWD) {
+    double z[C];
+    if (KIND == LAY_FWD_FIRST) {
+      first_layer<D, C>(p.W0, p.b0, k, q, beta, z);
+    } else {
+#pragma unroll
+      for (int c = 0; c < C; c++) z[c] = p.zin[(pt * C + c) * p.K + k];
+      z[0] += p.bias[k];
+    }
+    tanh_jet<D, C>(z, x);
+  } else {
+    if (KIND == LAY_REV_LAST) {
+      for (int f = 0; f < p.nf; f++) {
+        const double w = p.Wlast[f * p.K + k];
+#pragma unroll
+        for (int c = 0; c < C; c++) x[c] = fma(w, p.seeds[(item * p.nf + f) * CR + c], x[c]);
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < C; c++) x[c] = p.hbar[(item * C + c) * p.K + k];
+    }
+    double z[CR];
+#pragma unroll
+    for (int c = 1; c < CR; c++) z[c] = p.zin[(pt * p.cz + c) * p.K + k];
+    tanh_jet_adjoint<D>(p.hin[pt * CR * p.K + k], z, x);
+  }
+}
+
+// One element (a whole warp: component c of an item, output col) as an FP64 sum.  The operand is computed
+// again where it is not kept (forward).
+template <int D, int C, int KIND>
+__device__ __noinline__ double lay_exact(const LayArgs& p, int col, int64_t item, int c) {
+  const int lane = threadIdx.x & 31;
+  const int64_t pt = KIND <= LAY_FWD ? item : item / p.nr;
+  double sum = 0.0;
+#pragma unroll 1
+  for (int k = lane; k < p.K; k += 32) {
+    double a;
+    if constexpr (KIND <= LAY_FWD) {
+      double x[C];
+      const bool first = KIND == LAY_FWD_FIRST;
+      lay_operand<D, C, KIND>(p, item, pt, k, first ? p.qb[2 * pt] : 0.0, first ? p.qb[2 * pt + 1] : 0.0, x);
+      a = x[0];
+#pragma unroll
+      for (int i = 1; i < C; i++) a = i == c ? x[i] : a;
+    } else {
+      a = p.abar[(item * C + c) * p.K + k];   // (stored by this block before its last barrier)
+    }
+    sum = fma(a, p.W[col * p.wso + k * p.wsk], sum);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  return sum;
+}
+
 // One CTA per SM, persistent over tiles of 128 rows (128 / C items of C components).  Its 16 warps
 // first produce the tile's A operand, one item per warp: FP64 jets through tanh (or its adjoint),
-// the rows' exponents, their digits into shared memory in the layout the MMA reads.  One thread
-// then issues the 28 digit-pair products into seven tensor-memory accumulators of 64 columns, and
-// all warps combine the levels and store the layer's FP64 result.  The three phases follow one another:
-// the tile fills the shared memory (112 KB of A digits beside 56 KB of weights), and with the
-// FP64 pipe bound producer at 70-90 % of the time there is little to overlap.
+// the rows' exponents, their slices into shared memory in the layout the MMA reads.  One thread
+// then issues the 36 digit-pair products and that of the magnitudes into eight tensor-memory accumulators of
+// 64 columns, and all warps combine the levels and store the layer's FP64 result.  The three phases follow one
+// another: the tile fills the shared memory (144 KB of A beside 72 KB of weights) and the tensor memory.
 template <int D, int C, int KIND>
-__global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
+__global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const __grid_constant__ LayArgs p) {
   constexpr int CR = JT<D>::CR;
   constexpr int IPT = 128 / C;               // items per tile
   constexpr bool kFwd = KIND <= LAY_FWD;
@@ -273,12 +392,13 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
   __shared__ int eA[128], eW[kLayW];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int ks_n = (p.K + 31) >> 5;
-  for (int idx = t; idx < kLayS * kLayW * 8; idx += kLayThreads) {   // 16-byte chunks
+  for (int idx = t; idx < kLaySl * kLayW * 8; idx += kLayThreads) {   // 16-byte chunks
     const int s = idx / (kLayW * 8), row = (idx >> 3) % kLayW, c8 = idx & 7;
     *reinterpret_cast<uint4*>(Ws + s * kLayWSlice + swz(row, c8 * 8, kLayW)) =
         *reinterpret_cast<const uint4*>(p.wsl + (size_t)idx * 16);
   }
   if (t < kLayW) eW[t] = p.we[t];
+  const int ck[2] = {p.wc[lane], p.wc[lane + 32]};
   if (t == 0) {
     mbar_init(&done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -303,9 +423,9 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
       const int64_t item = i0 + it;
       const int64_t pt = kFwd ? item : item / p.nr;
       double x[2][C];
-      unsigned m[C];
+      int m[C];
 #pragma unroll
-      for (int c = 0; c < C; c++) m[c] = 0;
+      for (int c = 0; c < C; c++) m[c] = kLayZero;
       double q = 0.0, beta = 0.0;
       if (KIND == LAY_FWD_FIRST) {
         q = p.qb[2 * pt];
@@ -317,60 +437,40 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
 #pragma unroll
         for (int c = 0; c < C; c++) x[s][c] = 0.0;
         if (k >= p.K) continue;
+        lay_operand<D, C, KIND>(p, item, pt, k, q, beta, x[s]);
         if constexpr (kFwd) {
-          double z[C];
-          if (KIND == LAY_FWD_FIRST) {
-            first_layer<D, C>(p.W0, p.b0, k, q, beta, z);
-          } else {
-#pragma unroll
-            for (int c = 0; c < C; c++) z[c] = p.zin[(pt * C + c) * p.K + k];
-            z[0] += p.bias[k];
-          }
-          tanh_jet<D, C>(z, x[s]);
           if (p.hout) {
 #pragma unroll
             for (int c = 0; c < CR; c++) p.hout[(pt * CR + c) * p.K + k] = x[s][c];
           }
         } else {
-          if (KIND == LAY_REV_LAST) {
-            for (int f = 0; f < p.nf; f++) {
-              const double w = p.Wlast[f * p.K + k];
-#pragma unroll
-              for (int c = 0; c < C; c++) x[s][c] = fma(w, p.seeds[(item * p.nf + f) * CR + c], x[s][c]);
-            }
-          } else {
-#pragma unroll
-            for (int c = 0; c < C; c++) x[s][c] = p.hbar[(item * C + c) * p.K + k];
-          }
-          double z[CR];
-#pragma unroll
-          for (int c = 1; c < CR; c++) z[c] = p.zin[(pt * p.cz + c) * p.K + k];
-          tanh_jet_adjoint<D>(p.hin[pt * CR * p.K + k], z, x[s]);
 #pragma unroll
           for (int c = 0; c < C; c++) p.abar[(item * C + c) * p.K + k] = x[s][c];
         }
 #pragma unroll
         for (int c = 0; c < C; c++) {
-          const unsigned h = abs_hi(x[s][c]);
-          m[c] = h > m[c] ? h : m[c];
+          const int e = exponent_above(x[s][c], ck[s]);
+          m[c] = e > m[c] ? e : m[c];
         }
       }
 #pragma unroll
       for (int c = 0; c < C; c++) {
         const int row = it * C + c;
-        const int e = row_exponent(__reduce_max_sync(0xffffffffu, m[c]));
+        const int e = __reduce_max_sync(0xffffffffu, m[c]);
         if (lane == 0) {
           eA[row] = e;
-          if (kFwd && c < CR && p.hexp) p.hexp[pt * CR + c] = e;
+          if (kFwd && c < CR && p.hexp) p.hexp[pt * CR + c] = e == kLayZero ? 0 : e;
         }
 #pragma unroll
         for (int s = 0; s < 2; s++) {
           if (s < ks_n) {
-            const long long u = biased_digits(x[s][c], e == kLayBad ? 0 : e);
+            const int ek = e == kLayBad || e == kLayZero ? kNoDigits : e - ck[s];
+            const unsigned long long u = biased_digits(x[s][c], ek);
             unsigned char* dst = As + swz(row, lane + 32 * s, 128);
 #pragma unroll
             for (int d = 0; d < kLayS; d++)
               *reinterpret_cast<unsigned short*>(dst + d * kLayASlice) = digit_bf16(u, d);
+            *reinterpret_cast<unsigned short*>(dst + kLayS * kLayASlice) = magnitude_bf16(x[s][c], ek);
           }
         }
       }
@@ -381,17 +481,24 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
     // ---- products ----------------------------------------------------------------------------------
     if (t == 0) {
       tc_fence_after();
-      const uint32_t a0 = smem_u32(As), w0 = smem_u32(Ws);
+      // (four MMAs take about 128 clocks: one thread must not spend them on descriptors)
+      const uint64_t a0 = smem_desc(smem_u32(As)), w0 = smem_desc(smem_u32(Ws));
+      auto product = [&](int slot, int sa, int sw, uint32_t acc) {
+        const uint64_t a = a0 + (uint32_t)(sa * (kLayASlice >> 4)), w = w0 + (uint32_t)(sw * (kLayWSlice >> 4));
+        const uint32_t d = tmem + slot * kLayW;
+        mma_bf16<kLayW>(d, a, w, acc);
+        mma_bf16<kLayW>(d, a + 2, w + 2, 1);
+        if (ks_n > 1) {
+          mma_bf16<kLayW>(d, a + (128 * 64 >> 4), w + (kLayW * 64 >> 4), 1);
+          mma_bf16<kLayW>(d, a + (128 * 64 >> 4) + 2, w + (kLayW * 64 >> 4) + 2, 1);
+        }
+      };
+      product(7, kLayS, kLayS, 0);
 #pragma unroll 1
-      for (int slot = 0; slot < kLayS; slot++)
+      for (int level = kLayS - 1; level >= 0; level--)   // level 7 goes below level 6
 #pragma unroll 1
-        for (int s = 0; s <= slot; s++)
-          for (int ks = 0; ks < ks_n; ks++)
-#pragma unroll
-            for (int kk = 0; kk < 2; kk++)
-              mma_bf16<kLayW>(tmem + slot * kLayW, smem_desc(a0 + s * kLayASlice + ks * 128 * 64 + kk * 32),
-                              smem_desc(w0 + (slot - s) * kLayWSlice + ks * kLayW * 64 + kk * 32),
-                              (s == 0 && ks == 0 && kk == 0) ? 0u : 1u);
+        for (int s = 0; s <= level; s++)
+          product(level < 6 ? level : 6, s, level - s, (s == 0 && level != 6) ? 0u : 1u);
       mma_commit(&done);
     }
     // (read here: behind the next barrier the producers of the next tile overwrite the exponents)
@@ -422,19 +529,35 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const LayArgs p) {
         tmem_wait_ld();
 #pragma unroll
         for (int s = 0; s < kLayS; s++) tmem_use8(r[s]);
+        unsigned weak = 0;   // columns whose products are too small for their digits
 #pragma unroll
         for (int j = 0; j < 8; j++) {
-          const int col = col0 + j;
-          int v[kLayS];
+          int v[7];   // accumulator s is v_s 256^-s
 #pragma unroll
-          for (int s = 0; s < kLayS; s++) v[s] = __float2int_rn(__uint_as_float(r[s][j]));
-          // sum_s v_s 256^(5 - s), the last level rounded in: |.| < 2^61
-          const long long hi = (long long)v[0] * 65536 + (v[1] * 256 + v[2]);
-          const long long lo = (long long)v[3] * 65536 + (v[4] * 256 + v[5]);
-          const long long T = (hi << 24) + lo + ((v[6] + 128) >> 8);
-          const int ew = eW[col];
-          const double d = (ea == kLayBad || ew == kLayBad) ? nan("") : scaled_int(T, ea + ew - 54);
-          if (valid && col < p.N) p.out[orow * p.N + col] = d;
+          for (int s = 0; s < 7; s++)
+            v[s] = __float2int_rn(__uint_as_float(r[s][j]) * __uint_as_float(0x3f800000u + ((unsigned)s << 26)));
+          // sum_s v_s 256^(6 - s) = hi 2^24 + low, 0 <= low < 2^24, |hi| < 2^43; four bits of low go where hi is large
+          const long long lo = (long long)v[4] * 65536 + (v[5] * 256 + v[6]);
+          const long long hi = (long long)v[0] * 16777216 + (long long)v[1] * 65536 + (v[2] * 256 + v[3]) + (lo >> 24);
+          const unsigned low = (unsigned)lo & 0xffffffu;
+          const bool large = (unsigned long long)(hi + (1ll << 39)) >> 40;
+          const long long T = large ? hi * (1 << 20) + (low >> 4) : hi * (1 << 24) + low;
+          const int ew = eW[col0 + j];
+          const bool bad = ea == kLayBad || ew == kLayBad, zero = ea == kLayZero || ew == kLayZero;
+          const float S = __uint_as_float(r[7][j]);   // never above the true one
+          if (valid && col0 + j < p.N) {
+            p.out[orow * p.N + col0 + j] = zero ? 0.0 : scaled_int(T, ea + ew - (large ? 56 : 60));
+            if (bad || !(zero || S >= 0.04f)) weak |= 1u << j;   // 2^-4.64
+          }
+        }
+        if (__any_sync(0xffffffffu, weak)) {
+#pragma unroll 1
+          for (int j = 0; j < 8; j++)
+            for (unsigned b = __ballot_sync(0xffffffffu, weak >> j & 1); b; b &= b - 1) {
+              const int src = __ffs(b) - 1, rs = (warp & 3) * 32 + src;
+              const double v = lay_exact<D, C, KIND>(p, col0 + j, i0 + rs / C, rs % C);
+              if (lane == src) p.out[orow * p.N + col0 + j] = v;
+            }
         }
       }
     }
@@ -702,28 +825,6 @@ constexpr int kEntS = 8;
 constexpr int kEntASlice = 128 * 64, kEntBSlice = 64 * 64;   // K padded to 32: the layout of lay_gemm
 constexpr int kEntOps = kEntS * (kEntASlice + kEntBSlice);
 constexpr size_t kEntSmem = 1024 + kEntOps + 128 * 65 * 8;
-// digits of x 2^(62 - e): bytes 0..6 plus 128, then the signed top
-__device__ __forceinline__ long long biased_digits62(double x, int e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7ff);
-  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-  if (ex > 0) m |= 1ull << 52;
-  const int sh = (ex > 0 ? ex : 1) - 1013 - e;   // <= 9
-  unsigned long long v;
-  if (sh >= 0) v = sh > 9 ? 0ull : m << sh;
-  else v = sh < -54 ? 0ull : (m + (1ull << (-sh - 1))) >> -sh;
-  return ((b >> 63) ? -(long long)v : (long long)v) + 0x80808080808080ll;
-}
-__device__ __forceinline__ unsigned short digit62_bf16(long long u, int q) {
-  const unsigned lo = (unsigned)u, hi = (unsigned)((unsigned long long)u >> 32);
-  float f;
-  if (q == 0) f = (float)((int)hi >> 24);
-  else {
-    const int byte = 7 - q;   // 0..6
-    f = __uint_as_float(__byte_perm(byte < 4 ? lo : hi, 0x4B000000u, 0x7540 + (byte & 3))) - 8388736.0f;
-  }
-  return (unsigned short)(__float_as_uint(f) >> 16);
-}
 __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEntries p) {
   constexpr int CR = 6;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -803,10 +904,10 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEn
       const int r = t < 128 ? t : t - 128, stride = t < 128 ? kEntASlice : kEntBSlice;
 #pragma unroll
       for (int c = 0; c < CR; c++) {
-        const long long v = biased_digits62(x[c], bad ? 5000 : m - (t < 128 ? eh[c] : -eh[c]));
+        const unsigned long long v = biased_digits(x[c], bad ? kNoDigits : m - (t < 128 ? eh[c] : -eh[c]));
         unsigned char* dst = row + swz(r, c, 0);
 #pragma unroll
-        for (int d = 0; d < kEntS; d++) *reinterpret_cast<unsigned short*>(dst + d * stride) = digit62_bf16(v, d);
+        for (int d = 0; d < kEntS; d++) *reinterpret_cast<unsigned short*>(dst + d * stride) = digit_bf16(v, d);
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -844,7 +945,8 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEn
       for (int j = 0; j < 8; j++) {
         int v[kEntS];
 #pragma unroll
-        for (int s = 0; s < kEntS; s++) v[s] = __float2int_rn(__uint_as_float(r[s][j]));
+        for (int s = 0; s < kEntS; s++)   // (accumulator s is v_s 256^-s)
+          v[s] = __float2int_rn(__uint_as_float(r[s][j]) * __uint_as_float(0x3f800000u + ((unsigned)s << 26)));
         // sum_s v_s 256^(6 - s), the last level rounded in: below 2^63
         const long long hi = v[0] * 65536 + v[1] * 256 + v[2];
         const long long T = (hi << 32) + (long long)v[3] * 16777216 + (long long)v[4] * 65536 +
@@ -996,7 +1098,7 @@ int64_t lay_point_doubles(const NetDesc& net, int d, int nf, int ne, int mode) {
 }
 int64_t lay_ldg(const NetDesc& net) { return (net.P + 1 + 15) / 16 * 16; }
 int64_t lay_parts_doubles(const NetDesc& net) { return kLayParts * lay_ldg(net); }
-constexpr int64_t kLayFixed = 2 * GN_MAX_LAYERS * (kLayS * kLayW * kLayW * 2 + kLayW * 4) + 8192;   // weight slices
+constexpr int64_t kLayFixed = 2 * GN_MAX_LAYERS * (kLaySl * kLayW * kLayW * 2 + 2 * kLayW * 4) + 8192;   // weight slices
 
 int sm_count() {
   static const int n = [] {
@@ -1041,14 +1143,15 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
   const int ne = A.kind == KIND_INTERIOR ? NE : 1;
   const int nr = MODE == MODE_JACOBIAN ? ne : 1;
   unsigned char* wsl = static_cast<unsigned char*>(ws);
-  int* we = reinterpret_cast<int*>(wsl + (size_t)2 * (L - 2) * kLayS * kLayW * kLayW * 2);
+  int* we = reinterpret_cast<int*>(wsl + (size_t)2 * (L - 2) * kLaySl * kLayW * kLayW * 2);
+  int* wc = we + 2 * (L - 2) * kLayW;
   double* parts = reinterpret_cast<double*>(wsl + kLayFixed);
   double* buf = parts + lay_parts_doubles(net);
   int64_t chunk = (int64_t)((ws_bytes - kLayFixed) / 8 - lay_parts_doubles(net)) /
                   lay_point_doubles(net, D, NF, NE, MODE);
   const int64_t wave = (int64_t)sm_count() * (128 / C);   // points of one round of forward tiles
   if (chunk > 2 * wave) chunk = chunk / wave * wave;
-  const size_t opb = (size_t)kLayS * kLayW * kLayW * 2;
+  const size_t opb = (size_t)kLaySl * kLayW * kLayW * 2;
   for (int64_t p0 = A.pt0; p0 < A.pt1; p0 += chunk) {
     const int64_t n = p0 + chunk < A.pt1 ? chunk : A.pt1 - p0;
     double* at = buf;
@@ -1086,6 +1189,7 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
     pr.net = net;
     pr.wsl = wsl;
     pr.we = we;
+    pr.wc = wc;
     pr.pt_blocks = (int)((n + 255) / 256);
     const int wblocks = p0 == A.pt0 ? (L - 2) * 2 * kLayW / 8 : 0;   // the weights once per pass
     lay_inputs<D><<<pr.pt_blocks + wblocks, 256, 0, st>>>(pr);
@@ -1113,6 +1217,10 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
       g.out = Z[j + 1];
       g.wsl = wsl + (size_t)(2 * (j - 1)) * opb;
       g.we = we + 2 * (j - 1) * kLayW;
+      g.wc = wc + 2 * (j - 1) * kLayW;
+      g.W = A.theta + net.offW[j];
+      g.wso = net.w[j];
+      g.wsk = 1;
       e = j == 1 ? run_gemm<D, C, LAY_FWD_FIRST>(g, st) : run_gemm<D, C, LAY_FWD>(g, st);
     }
     if (e != cudaSuccess) return e;
@@ -1141,6 +1249,10 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
       g.out = hb[j & 1];
       g.wsl = wsl + (size_t)(2 * (j - 1) + 1) * opb;
       g.we = we + (2 * (j - 1) + 1) * kLayW;
+      g.wc = wc + (2 * (j - 1) + 1) * kLayW;
+      g.W = A.theta + net.offW[j];
+      g.wso = 1;
+      g.wsk = net.w[j];
       e = j == L - 2 ? run_gemm<D, CR, LAY_REV_LAST>(g, st) : run_gemm<D, CR, LAY_REV>(g, st);
       if (e != cudaSuccess) return e;
       hbar = hb[j & 1];

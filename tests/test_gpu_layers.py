@@ -169,3 +169,60 @@ def test_tiles_keep_their_own_exponents(name, hidden, n):
     assert rel(host(first[sel]), ref) <= TOL
     for _ in range(5):
         assert torch.equal(pb.residual(th, big.lam)[0], first)
+
+
+def _neuron(theta, widths, layer, k, s):
+    """Incoming weights of a hidden neuron divided by s, outgoing ones multiplied."""
+    off = 0
+    for l, (i, o) in enumerate(zip(widths[:-1], widths[1:])):
+        W = theta[off:off + i * o].reshape(o, i)
+        if l == layer - 1:
+            W[k] /= s
+        elif l == layer:
+            W[:, k] *= s
+        off += i * o + o
+
+
+def _wild(theta, widths, rng):
+    """Hidden-to-hidden weights spread over five decades, which no scaling of neurons evens out."""
+    off = 0
+    for l, (i, o) in enumerate(zip(widths[:-1], widths[1:])):
+        if 0 < l < len(widths) - 2:
+            theta[off:off + i * o] *= 10.0 ** rng.uniform(-4.5, 0.5, i * o)
+        off += i * o + o
+
+
+@pytest.mark.parametrize("name,hidden", [("ipm", [64, 64, 64, 64]), ("burgers", [40, 40, 40]), ("boussinesq", [56, 60, 64])])
+@pytest.mark.parametrize("scales", [1e2, 1e4, 1e6, 1e-5, "wild"])
+def test_weights_of_different_scale(name, hidden, scales):
+    """Rows and Jacobian columns as accurate as FP64 sums when a network's weights differ in scale.  An
+    FP64 sum of n <= 64 products is the exact sum of operands off by at most n 2^-53 each, so what
+    such changes of theta move bounds what two FP64 evaluations may differ by (times 4, for
+    the layers' changes that do not point the same way)."""
+    n = 4200
+    big, few, pick, pb, pf = _pair(name, hidden, n)
+    ne = EQS[name][1]
+    rng = np.random.default_rng(8)
+    theta = big.theta.copy()
+    if scales == "wild":
+        _wild(theta, big.widths, rng)
+    else:
+        for layer in range(1, len(hidden)):
+            _neuron(theta, big.widths, layer, 5 + layer, scales)
+    m = len(pick) * ne
+    sel = torch.from_numpy(_rows(pick, ne)).cuda()
+    s = np.sqrt(len(pick) / n)
+
+    def few_at(th):
+        return s * host(pf.residual(dev(th), big.lam)[0][:m]), s * host(pf.jacobian(dev(th), big.lam)[:m])
+
+    r0, J0 = few_at(theta)
+    tr, tJ = 0.0, np.zeros(J0.shape[1])
+    for _ in range(4):
+        r, J = few_at(theta * (1.0 + 64 * 2.0 ** -53 * rng.uniform(-1, 1, theta.size)))
+        tr = max(tr, np.max(np.abs(r - r0)))
+        tJ = np.maximum(tJ, np.max(np.abs(J - J0), axis=0))
+    th = dev(theta)
+    assert np.max(np.abs(host(pb.residual(th, big.lam)[0][sel]) - r0)) <= 4 * tr
+    dJ = np.max(np.abs(host(pb.jacobian(th, big.lam)[sel]) - J0), axis=0)
+    assert np.all(dJ <= 4 * tJ + 2.0 ** -48 * np.max(np.abs(J0), axis=0))
