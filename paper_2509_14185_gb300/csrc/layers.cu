@@ -814,17 +814,25 @@ __global__ void __launch_bounds__(256) lay_entries(const LayEntries p) {
 // (rows x out) x 6 x in contraction per point and layer, whose FP64 form (lay_entries) bounds the 2D
 // Jacobian.  One CTA per SM, persistent over (point, layer, pair of rows): 128 x 64 outputs, K = 6 of 16.
 // A component's scale moves between the factors by powers of two (h_c is taken relative to its own
-// largest element 2^eh_c, abar_c times that); then every output row and column has one exponent over
-// its six terms.  62-bit integers in eight digits (nine bits below FP64's last for the row's largest
-// term), the 36 digit pairs of the eight leading levels summed exactly: an entry's error stays below
-// that of the FP64 sum unless all its terms lie 2^9 under the product of its row's and its column's largest.
+// row's exponent 2^eh_c, abar_c times that); then every output row and column has one exponent over
+// its six terms.  62-bit integers in eight digits and the 36 digit pairs of the eight leading levels, as in
+// lay_gemm; what is dropped is at most 6 * 2^-58.99 2^(e_a + e_b) and the last level's rounding 2^-61 of that unit, which is
+// within the 6 * 2^-53 S of the FP64 sum wherever S >= 2^-5.9 2^(e_a + e_b), S the sum of the six products'
+// magnitudes.  S comes from FP32 forms of the operands; an entry below that line (Xavier weights, 4 x 64:
+// 0.05 to 0.4 % of them), or with a factor that is not finite, is summed in FP64.  (Its operands stay in shared
+// memory for that: a warp in sixteen has such an entry, and all wait for the slowest.)
 // Bound by the digits and the 64-bit recombination (integer pipes) and by J's stores.
 // Jacobian of 32,768 IPM rows, four hidden layers of 64: 6.96 -> 5.54 ms.  Digits dealt over all threads
 // (5.64 ms) and stores of the unit before beside the products (5.67 ms) were no faster.
 constexpr int kEntS = 8;
 constexpr int kEntASlice = 128 * 64, kEntBSlice = 64 * 64;   // K padded to 32: the layout of lay_gemm
 constexpr int kEntOps = kEntS * (kEntASlice + kEntBSlice);
-constexpr size_t kEntSmem = 1024 + kEntOps + 128 * 65 * 8;
+constexpr int kEntLd = 7;   // doubles per operand row of the FP64 sums
+constexpr size_t kEntSmem = 1024 + kEntOps + 128 * 65 * 8 + 192 * kEntLd * 8;
+// (a call: predicated, its FP64 instructions would take their slots for every entry, 9.0 ms instead of 5.7 for the Jacobian above)
+__device__ __noinline__ double entry_sum(const double* a, const double* h) {
+  return fma(a[2], h[2], fma(a[1], h[1], a[0] * h[0])) + fma(a[5], h[5], fma(a[4], h[4], a[3] * h[3]));
+}
 __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEntries p) {
   constexpr int CR = 6;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -832,9 +840,12 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEn
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char* Bs = As + kEntS * kEntASlice;
   double* out_tile = reinterpret_cast<double*>(As + kEntOps);   // [128][65]
+  double* xs = out_tile + 128 * 65;                             // [192][kEntLd]: the operand rows themselves
   __shared__ uint64_t done;
   __shared__ uint32_t tmem_slot;
   __shared__ int eA[128], eB[64];
+  __shared__ float fA[128][7];                  // |factors| relative to 2^eA, 2^eB (pitch 7: no bank conflicts)
+  __shared__ __align__(16) float fB[64][8];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   for (int idx = t; idx < kEntOps / 16; idx += kLayThreads)   // components 6 .. 31 stay zero
     reinterpret_cast<uint4*>(As)[idx] = make_uint4(0, 0, 0, 0);
@@ -888,26 +899,25 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEn
     const int l = 1 + (int)(u / ng % nl), g = (int)(u % ng);
     const int in = p.net.w[l], out = p.net.w[l + 1];
     if (t < 192) {
-      int m = -100000;
-      bool bad = false;
+      int m = kLayZero;
 #pragma unroll
       for (int c = 0; c < CR; c++) {
-        const int ex = (int)(abs_hi(x[c]) >> 20);
-        bad = bad || ex == 0x7ff || eh[c] == kLayBad;
-        const int e = (ex > 0 ? ex : 1) - 1022 + (t < 128 ? eh[c] : -eh[c]);
-        if (x[c] != 0.0) m = e > m ? e : m;
+        const int e = eh[c] == kLayBad ? kLayBad : exponent_above(x[c], t < 128 ? eh[c] : -eh[c]);
+        m = e > m ? e : m;
       }
-      if (m == -100000) m = 0;
-      if (t < 128) eA[t] = bad ? kLayBad : m;
-      else eB[t - 128] = bad ? kLayBad : m;
+      (t < 128 ? eA[t] : eB[t - 128]) = m;
+      const bool none = m == kLayBad || m == kLayZero;
       unsigned char* row = t < 128 ? As : Bs;
       const int r = t < 128 ? t : t - 128, stride = t < 128 ? kEntASlice : kEntBSlice;
 #pragma unroll
       for (int c = 0; c < CR; c++) {
-        const unsigned long long v = biased_digits(x[c], bad ? kNoDigits : m - (t < 128 ? eh[c] : -eh[c]));
+        const unsigned long long v = biased_digits(x[c], none ? kNoDigits : m - (t < 128 ? eh[c] : -eh[c]));
         unsigned char* dst = row + swz(r, c, 0);
 #pragma unroll
         for (int d = 0; d < kEntS; d++) *reinterpret_cast<unsigned short*>(dst + d * stride) = digit_bf16(v, d);
+        const float f = (float)abs((int)((long long)(v - kDigitBias) >> 32)) * 0x1p-30f;
+        (t < 128 ? fA[t][c] : fB[t - 128][c]) = f;
+        xs[t * kEntLd + c] = x[c];
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -915,13 +925,13 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEn
     __syncthreads();
     if (t == 0) {
       tc_fence_after();
-      const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
-#pragma unroll 1
+      const uint64_t a0 = smem_desc(smem_u32(As)), b0 = smem_desc(smem_u32(Bs));
+#pragma unroll
       for (int slot = 0; slot < kEntS; slot++)
-#pragma unroll 1
+#pragma unroll
         for (int s = 0; s <= slot; s++)
-          mma_bf16<64>(tmem + slot * 64, smem_desc(a0 + s * kEntASlice), smem_desc(b0 + (slot - s) * kEntBSlice),
-                       s == 0 ? 0u : 1u);
+          mma_bf16<64>(tmem + slot * 64, a0 + (uint32_t)(s * (kEntASlice >> 4)),
+                       b0 + (uint32_t)((slot - s) * (kEntBSlice >> 4)), s == 0 ? 0u : 1u);
       mma_commit(&done);
     }
     load(u + gridDim.x);   // arrives beside the products and the stores
@@ -930,6 +940,10 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEn
     if (!ok) break;   // the host sees the status bit
     tc_fence_after();
     const int row = (warp & 3) * 32 + lane, ea = eA[row];
+    const int re = 2 * g + (row >> 6), ro = row & 63;   // this row's residual row and output
+    float fa[CR];
+#pragma unroll
+    for (int c = 0; c < CR; c++) fa[c] = fA[row][c];
 #pragma unroll 1
     for (int part = 0; part < 2; part++) {
       const int col0 = (warp >> 2) * 16 + part * 8;
@@ -941,6 +955,7 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEn
       tmem_wait_ld();
 #pragma unroll
       for (int s = 0; s < kEntS; s++) tmem_use8(r[s]);
+      unsigned weak = 0;
 #pragma unroll
       for (int j = 0; j < 8; j++) {
         int v[kEntS];
@@ -951,8 +966,18 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEn
         const long long hi = v[0] * 65536 + v[1] * 256 + v[2];
         const long long T = (hi << 32) + (long long)v[3] * 16777216 + (long long)v[4] * 65536 +
                             (v[5] * 256 + v[6] + ((v[7] + 128) >> 8));
-        const int eb = eB[col0 + j];
-        out_tile[row * 65 + col0 + j] = (ea == kLayBad || eb == kLayBad) ? nan("") : scaled_int(T, ea + eb - 60);
+        const int i = col0 + j, eb = eB[i];
+        const bool bad = ea == kLayBad || eb == kLayBad, zero = ea == kLayZero || eb == kLayZero;
+        out_tile[row * 65 + i] = zero ? 0.0 : scaled_int(T, ea + eb - 60);
+        const float4 b4 = *reinterpret_cast<const float4*>(&fB[i][0]);
+        const float2 b2 = *reinterpret_cast<const float2*>(&fB[i][4]);
+        const float S = fmaf(fa[0], b4.x, fmaf(fa[1], b4.y, fmaf(fa[2], b4.z, fmaf(fa[3], b4.w, fmaf(fa[4], b2.x, fa[5] * b2.y)))));
+        if (bad || (!zero && S < 0.017f)) weak |= 1u << j;   // 2^-5.88
+      }
+      if (re >= p.nr || ro >= out) weak = 0;
+      for (; weak; weak &= weak - 1) {   // every lane its own entries
+        const int i = col0 + __ffs(weak) - 1;
+        if (i < in) out_tile[row * 65 + i] = entry_sum(xs + row * kEntLd, xs + (128 + i) * kEntLd);
       }
     }
     tc_fence_before();

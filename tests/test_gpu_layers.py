@@ -226,3 +226,29 @@ def test_weights_of_different_scale(name, hidden, scales):
     assert np.max(np.abs(host(pb.residual(th, big.lam)[0][sel]) - r0)) <= 4 * tr
     dJ = np.max(np.abs(host(pb.jacobian(th, big.lam)[sel]) - J0), axis=0)
     assert np.all(dJ <= 4 * tJ + 2.0 ** -48 * np.max(np.abs(J0), axis=0))
+
+
+@pytest.mark.parametrize("name,hidden", [("ipm", [48, 64, 48, 45]), ("boussinesq", [56, 64, 60])])
+def test_entries_of_a_constant_neuron(name, hidden):
+    """A hidden neuron without incoming weights is h = tanh(b): its outgoing weight's entry is h times the
+    entry of the bias behind it, in every row, however small beside the row's other entries.
+    Of the FP64 sum's six terms one is not 0: off by 6 u at most, tanh by 2 ulp (4 u) on
+    either side, the product here by u."""
+    eq, nf = EQS[name]
+    n = 8000
+    w = I.weighted(I.small_case(eq, [2] + hidden + [nf], n, n_bnd=0, seed=5))
+    theta, offs, off = w.theta.copy(), [], 0
+    for i, o in zip(w.widths[:-1], w.widths[1:]):
+        offs.append((off, i, o))
+        off += i * o + o
+    b = 0.7
+    for off, i, o in offs[:-2]:
+        theta[off + 3 * i:off + 4 * i] = 0.0
+        theta[off + i * o + 3] = b
+    pb = gpu_problem(w)
+    J = pb.jacobian(dev(theta), w.lam)[:n * EQS[name][1]]
+    for off, i, o in offs[1:-1]:
+        entry, bias = J[:, off + 3:off + i * o:i], J[:, off + i * o:off + i * o + o]
+        ref = bias * np.tanh(b)
+        assert bool((ref != 0).any())
+        assert bool(((entry - ref).abs() <= 15 * 2.0 ** -53 * ref.abs()).all())
