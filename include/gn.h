@@ -54,7 +54,11 @@ extern "C" {
 #define GN_ERR_OOM           -3   /* device allocation failed */
 #define GN_ERR_NONFINITE     -4   /* a residual or loss was NaN or infinite */
 #define GN_ERR_NOT_SPD       -5   /* G + gamma I not positive definite after 5 damping escalations */
-#define GN_ERR_TIMEOUT       -6   /* a bounded device-side wait gave up */
+#define GN_ERR_TIMEOUT       -6   /* a bounded device-side wait gave up, in this call or in one before it on
+                                     the handle that did not synchronise (gn_jacobian, gn_gradient,
+                                     gn_residual without a loss: its results are not to be used).
+                                     Reported once, by gn_residual with a loss that is not finite, the
+                                     maximum residuals, gn_gram in split precision, gn_damped_solve and the steps */
 #define GN_ERR_UNSUPPORTED   -7   /* requested precision/path not available on this device */
 #define GN_ERR_TOO_LARGE     -8   /* size exceeds the fixed scratch of gn_jtr_noalloc (16384 columns) */
 #define GN_ERR_IO            -9   /* a checkpoint file could not be written or read */
@@ -489,12 +493,12 @@ int gn_jtr_noalloc(const double* J, int64_t ld, int64_t nrows, int64_t ncols, co
                    void* cuda_stream);
 
 /* Testing hook of the failure path GN_ERR_TIMEOUT (no paper counterpart).  Every wait of the
- * split-precision tensor-core kernels on an mbarrier (a copy landing, an MMA completing, an
+ * tensor-core kernels (split precision, and the passes over many points) on an mbarrier (a copy landing, an MMA completing, an
  * accumulator becoming free) is bounded in time; when one runs out, the kernel raises a
  * status bit, lets its copies and MMAs in flight finish (again with a bound), releases its
  * tensor memory and returns, and the calling entry point returns GN_ERR_TIMEOUT with the
  * CUDA context still usable.  wait_ns sets that bound for later launches (0 restores the
- * default of 4 s); starve_copies != 0 makes the kernels' producer issue no copies at all,
+ * default of 4 s); starve_copies != 0 makes the kernels issue no copies or, where none are, no MMAs,
  * so no copy or MMA is ever in flight and every consumer's wait runs out after wait_ns,
  * which lets a test exercise the path without any fault.  Process-wide; not for use while
  * other threads launch work.  Returns GN_OK. */

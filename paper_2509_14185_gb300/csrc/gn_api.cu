@@ -435,6 +435,22 @@ int max_res_of(gn_handle* h, const double* r) {
   return GN_OK;
 }
 
+// Status bit 1 of the word h->flag[2]: a bounded wait of a tensor-core kernel ran out.  Calls that only
+// launch work leave it standing; the next call that synchronises anyway reports and clears it.
+int timed_out(gn_handle* h, int word) {
+  if (!(word & 2)) return GN_OK;
+  GN_TRY_CUDA(cudaMemsetAsync(h->flag + 2, 0, sizeof(int), h->st));
+  set_detail(__FILE__, __LINE__, "a bounded wait in a tensor-core kernel timed out");
+  return GN_ERR_TIMEOUT;
+}
+int synchronise(gn_handle* h) {   // the handle's stream, with that report
+  GN_TRY_CUDA(cudaMemcpyAsync(&h->hpin[9], h->flag + 2, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+  GN_TRY_CUDA(cudaStreamSynchronize(h->st));
+  int f = 0;
+  memcpy(&f, &h->hpin[9], sizeof(int));
+  return timed_out(h, f);
+}
+
 int residual_loss(gn_handle* h, const double* theta, double lam, double* r, double* loss) {
   Pass ps = {MODE_RESIDUAL, r, nullptr, 0, 0, 0, nullptr};
   int rc = run_pass(h, theta, lam, ps, nullptr);
@@ -445,6 +461,8 @@ int residual_loss(gn_handle* h, const double* theta, double lam, double* r, doub
     GN_TRY_CUDA(cudaMemcpyAsync(h->hpin, h->red + 256, sizeof(double), cudaMemcpyDeviceToHost, h->st));
     GN_TRY_CUDA(cudaStreamSynchronize(h->st));
     *loss = 0.5 * h->hpin[0];
+    // the rows of a pass whose wait ran out are NaN, so a finite loss needs no look at the status
+    if (!std::isfinite(*loss)) return synchronise(h);
   }
   return GN_OK;
 }
@@ -784,14 +802,9 @@ int gn_gram(gn_handle* h, const double* J, int64_t ld, int64_t nrows, const doub
   if (precision < GN_PREC_FP64 || precision > GN_PREC_SPLIT_ALL) return GN_ERR_INVALID;
   if (precision == GN_PREC_FP64) return gram_into(h, J, ld, nrows, r, G_out, g_out, precision, accumulate);
   // split precision: report a timed-out tensor-core wait before returning
-  GN_TRY_CUDA(cudaMemsetAsync(h->flag + 2, 0, sizeof(int), h->st));
   int rc = gram_into(h, J, ld, nrows, r, G_out, g_out, precision, accumulate);
   if (rc) return rc;
-  GN_TRY_CUDA(cudaMemcpyAsync(&h->hpin[9], h->flag + 2, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-  GN_TRY_CUDA(cudaStreamSynchronize(h->st));
-  int f = 0;
-  memcpy(&f, &h->hpin[9], sizeof(int));
-  return (f & 2) ? GN_ERR_TIMEOUT : GN_OK;
+  return synchronise(h);
 }
 
 namespace {
@@ -818,10 +831,7 @@ int damped_solve(gn_handle* h, const double* G, const double* g, double* gamma, 
     GN_TRY_CUDA(cudaMemcpyAsync(&h->hpin[8], h->flag, 3 * sizeof(int), cudaMemcpyDeviceToHost, h->st));
     GN_TRY_CUDA(cudaStreamSynchronize(h->st));
     memcpy(hflag, &h->hpin[8], 3 * sizeof(int));
-    if (hflag[2] & 2) {
-      set_detail(__FILE__, __LINE__, "a bounded wait in a tensor-core kernel timed out");
-      return GN_ERR_TIMEOUT;
-    }
+    if (int rc = timed_out(h, hflag[2])) return rc;
     if (check_rows && (hflag[0] & 1)) return GN_ERR_NONFINITE;
     if (!hflag[1]) break;
     if (retries == 5) {
@@ -858,7 +868,7 @@ int gn_max_residual(gn_handle* h, const double* theta, double lambda, double* ou
   GN_TRY_CUDA(max_abs_rows(h->r, nint, 0, h->red, h->st));
   GN_TRY_CUDA(finish_max(h->red, h->red + 300, h->st));
   GN_TRY_CUDA(cudaMemcpyAsync(h->hpin, h->red + 300, sizeof(double), cudaMemcpyDeviceToHost, h->st));
-  GN_TRY_CUDA(cudaStreamSynchronize(h->st));
+  if ((rc = synchronise(h))) return rc;
   const double w = nint > 0 ? sqrt(2.0 / ((double)h->p.n_pts * h->ne)) : 1.0;
   *out = h->hpin[0] / w * (h->staged ? h->stage_eps : 1.0);   // stage 2: max |R| of Phi_1 + eps Phi_2
   return GN_OK;
@@ -874,9 +884,9 @@ int gn_step(gn_handle* h, double* theta, double* lambda, double* damping, gn_ste
   double gamma = *damping;
   Timer tm(st);
   Phases ph;
-  // status bits: [0] non-finite residual rows of this step's passes, [2] a timed-out wait
+  // status bits: [0] non-finite residual rows of this step's passes ([2], a timed-out wait, stands until
+  // it is reported)
   GN_TRY_CUDA(cudaMemsetAsync(h->flag, 0, sizeof(int), st));
-  GN_TRY_CUDA(cudaMemsetAsync(h->flag + 2, 0, sizeof(int), st));
   tm.mark(0);
   // 1. rows and Jacobian, Gram and gradient, streamed in row blocks
   int rc = GN_OK;
@@ -1023,7 +1033,6 @@ int gn_step_ema(gn_handle* h, double* theta, double* lambda, double* damping, do
   double* Jv = JD + R;   // J~ v_prev
   Timer tm(st);
   GN_TRY_CUDA(cudaMemsetAsync(h->flag, 0, sizeof(int), st));
-  GN_TRY_CUDA(cudaMemsetAsync(h->flag + 2, 0, sizeof(int), st));
   tm.mark(0);
   // 1. rows and the Jacobian
   Pass ps = {MODE_JACOBIAN, h->r, h->J, h->ldJ, 0, R, nullptr};
@@ -1089,7 +1098,10 @@ int gn_step_ema(gn_handle* h, double* theta, double* lambda, double* damping, do
   GN_TRY_CUDA(ema_update(theta, h->delta, v_prev, alpha, mu, P, Pp, h->theta_t, st));
   double ht = 0.0;
   rc = residual_loss(h, h->theta_t, lam_t, h->r, &ht);
-  if (rc) return rc;
+  if (rc) {   // v_prev holds a step that was not taken
+    GN_TRY_CUDA(cudaMemsetAsync(v_prev, 0, Pp * sizeof(double), st));
+    return rc;
+  }
   tm.mark(4);
   const double Jd2 = alpha * alpha * s[0] - 2.0 * alpha * mu * s[1] + mu * mu * s[2];
   const double model = alpha * g_d + mu * g_v + 0.5 * Jd2;   // undamped model change

@@ -250,6 +250,8 @@ int gram_split_choice(int S, int64_t Pp, int64_t nrows);
 int gram_tile_choice(int S, int64_t Pp, int64_t nrows);
 cudaError_t ensure_chol_streams(gn_handle* h);
 void graph_release(gn_handle* h);
+// wait for the handle's stream; GN_ERR_TIMEOUT if a bounded wait has run out since the last report
+int synchronise(gn_handle* h);
 
 // ---- launchers (host functions implemented in the .cu files) -----------
 cudaError_t launch_transpose_weights(const NetDesc& net, const double* theta, double* wt, cudaStream_t st);

@@ -87,7 +87,7 @@ namespace {
 // Model scalars after the solve (red[256] = |r~|^2, red[257] = g.delta, red[258] =
 // delta.G.delta, delta[P] = the lambda component); decides whether the line search runs.
 __global__ void model_kernel(const double* __restrict__ red, const double* __restrict__ delta, int64_t P,
-                             const int* __restrict__ flag, StepState* s, cudaGraphConditionalHandle first) {
+                             int* flag, StepState* s, cudaGraphConditionalHandle first) {
   s->n_trials = 0;
   s->accepted = 0;
   s->alpha = 1.0;
@@ -100,7 +100,9 @@ __global__ void model_kernel(const double* __restrict__ red, const double* __res
   s->dlam = delta[P];
   s->max_res = red[kMaxResSlot];
   int status = GN_OK;
-  if (flag[2] & 2) status = GN_ERR_TIMEOUT;          // a bounded tensor-core wait gave up
+  const bool late = flag[2] & 2;
+  flag[2] = 0;                                       // (reported)
+  if (late) status = GN_ERR_TIMEOUT;                 // a bounded tensor-core wait gave up
   else if (!isfinite(s->h0)) status = GN_ERR_NONFINITE;   // before the pivots: no retries on NaN rows
   else if (flag[1]) status = kNeedRetry;             // a pivot was not positive
   s->status = status;
@@ -119,8 +121,14 @@ __global__ void trial_kernel(const double* __restrict__ theta, const double* __r
 
 // Armijo test of the trial just evaluated (c1 = 1e-4, alpha halved after a rejection);
 // `next` is the condition of the following trial's IF node (none after the last trial).
-__global__ void armijo_kernel(const double* __restrict__ red, StepState* s, cudaGraphConditionalHandle next,
-                              int has_next) {
+__global__ void armijo_kernel(const double* __restrict__ red, int* flag, StepState* s,
+                              cudaGraphConditionalHandle next, int has_next) {
+  if (flag[2] & 2) {   // the trial's rows are not to be had: no step, no further trial
+    flag[2] = 0;
+    s->status = GN_ERR_TIMEOUT;
+    if (has_next) cudaGraphSetConditional(next, 0u);
+    return;
+  }
   const double ht = 0.5 * red[256];
   const double alpha = s->alpha;
   s->n_trials = s->n_trials + 1;
@@ -173,7 +181,6 @@ int mark(gn_handle* h, bool on, int k) {
 int capture_rows_gram(gn_handle* h, const double* theta, bool marks) {
   GraphState* gs = h->gs;
   cudaStream_t st = h->st;
-  GN_G_TRY(cudaMemsetAsync(h->flag + 2, 0, sizeof(int), st));
   const int64_t nblk = (h->n_rows + h->jrows - 1) / h->jrows;
   marks = marks && nblk == 1;
   int rc = mark(h, marks, 0);
@@ -271,7 +278,7 @@ int capture_solve(gn_handle* h, double* theta, bool marks, const cudaEvent_t* ga
     if (!rc) rc = loss_of(h, h->r, 0);
     if (!rc) {
       const bool has_next = t + 1 < kMaxTrials;
-      armijo_kernel<<<1, 1, 0, gs->body>>>(h->red, ds, has_next ? cond[t + 1] : cond[t], has_next ? 1 : 0);
+      armijo_kernel<<<1, 1, 0, gs->body>>>(h->red, h->flag, ds, has_next ? cond[t + 1] : cond[t], has_next ? 1 : 0);
       count_launch();
       if (GN_NOTE(cudaGetLastError()) != cudaSuccess) rc = GN_ERR_CUDA;
     }
@@ -296,7 +303,6 @@ int capture_solve(gn_handle* h, double* theta, bool marks, const cudaEvent_t* ga
 int capture_pipelined(gn_handle* h, double* theta, bool marks, int64_t chunk) {
   GraphState* gs = h->gs;
   cudaStream_t st = h->st;
-  GN_G_TRY(cudaMemsetAsync(h->flag + 2, 0, sizeof(int), st));
   int rc = mark(h, marks, 0);
   Pass ps = {MODE_JACOBIAN, h->r, h->J, h->ldJ, 0, h->n_rows, nullptr, &gs->ds->lam};
   if (!rc) rc = run_pass(h, theta, 0.0, ps, nullptr);

@@ -172,7 +172,7 @@ int gn_signed_max_residual(gn_handle* h, const double* theta, double lambda, dou
   count_launch();
   GN_L_TRY(cudaGetLastError());
   GN_L_TRY(cudaMemcpyAsync(h->hpin + 42, slot, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->st));
-  GN_L_TRY(cudaStreamSynchronize(h->st));
+  if ((rc = synchronise(h))) return rc;
   *r_hat = h->hpin[42];
   if (point) *point = (int64_t)h->hpin[43];
   return GN_OK;

@@ -74,6 +74,7 @@ struct LayArgs {
   int64_t wso, wsk;
   int* flag;
   unsigned long long wait_ns;
+  int starve;               // testing: no product is issued, so the waits run out
 };
 
 // tanh jets at one neuron: h[0..C) from the preactivation components z[0..C)
@@ -479,7 +480,7 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const __grid_constant
     tc_fence_before();
     __syncthreads();
     // ---- products ----------------------------------------------------------------------------------
-    if (t == 0) {
+    if (t == 0 && !p.starve) {
       tc_fence_after();
       // (four MMAs take about 128 clocks: one thread must not spend them on descriptors)
       const uint64_t a0 = smem_desc(smem_u32(As)), w0 = smem_desc(smem_u32(Ws));
@@ -510,6 +511,7 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_gemm(const __grid_constant
         for (int64_t i = tile * IPT * C * p.N + t; i < (tile + 1) * IPT * C * p.N && i < p.items * C * p.N;
              i += kLayThreads)
           p.out[i] = nan("");
+      mbar_wait(&done, phase ^ 1, p.flag, p.wait_ns);   // products in flight use the tensor memory to be released
       break;
     }
     tc_fence_after();
@@ -755,6 +757,7 @@ struct LayEntries {
   int hidden;                              // 0: the hidden-to-hidden weights are lay_hidden_entries'
   int* flag;
   unsigned long long wait_ns;
+  int starve;
 };
 // One warp per (point, layer): the layer's activation jets stay in registers (two neurons per
 // lane) for all rows of the point, the adjoints are read at one address per warp, consecutive lanes
@@ -923,7 +926,7 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEn
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
-    if (t == 0) {
+    if (t == 0 && !p.starve) {
       tc_fence_after();
       const uint64_t a0 = smem_desc(smem_u32(As)), b0 = smem_desc(smem_u32(Bs));
 #pragma unroll
@@ -937,7 +940,18 @@ __global__ void __launch_bounds__(kLayThreads, 1) lay_hidden_entries(const LayEn
     load(u + gridDim.x);   // arrives beside the products and the stores
     const bool ok = __syncthreads_and(mbar_wait(&done, phase, p.flag, p.wait_ns));
     phase ^= 1;
-    if (!ok) break;   // the host sees the status bit
+    if (!ok) {   // the host sees the status bit; this CTA's remaining entries become NaN
+      mbar_wait(&done, phase ^ 1, p.flag, p.wait_ns);   // (products in flight, as in lay_gemm)
+      for (; u < units; u += gridDim.x)
+        for (int r = warp; r < 128; r += kLayThreads / 32) {
+          const int ul = 1 + (int)(u / ng % nl), e = 2 * (int)(u % ng) + (r >> 6), o = r & 63, ui = p.net.w[ul];
+          const int64_t jr = p.row0 + (p.p0 + u / (nl * ng)) * p.nr + e;
+          if (e >= p.nr || o >= p.net.w[ul + 1] || jr < p.jlo || jr >= p.jhi) continue;
+          double* dst = p.J + (jr - p.jlo) * p.ldJ + p.net.offW[ul] + (int64_t)o * ui;
+          for (int i = lane; i < ui; i += 32) dst[i] = nan("");
+        }
+      break;
+    }
     tc_fence_after();
     const int row = (warp & 3) * 32 + lane, ea = eA[row];
     const int re = 2 * g + (row >> 6), ro = row & 63;   // this row's residual row and output
@@ -1230,6 +1244,7 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
     g.Wlast = A.theta + net.offW[L - 1];
     g.flag = A.flag + 2;
     g.wait_ns = g_oz_wait_ns.load(std::memory_order_relaxed);
+    g.starve = g_oz_starve.load(std::memory_order_relaxed);
     cudaError_t e = cudaSuccess;
     for (int j = 1; j <= L - 2 && e == cudaSuccess; j++) {
       g.items = n;
@@ -1311,6 +1326,7 @@ cudaError_t layers_eq(const JetArgs& A, void* ws, size_t ws_bytes, cudaStream_t 
     en.J = A.J;
     en.flag = A.flag + 2;
     en.wait_ns = g.wait_ns;
+    en.starve = g.starve;
     en.hidden = !hidden_entries<D>(net, nr);
     for (int j = 1; j < L; j++) en.He[j] = He[j];
     if (MODE == MODE_GRADIENT) {

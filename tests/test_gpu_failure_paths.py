@@ -96,3 +96,59 @@ def test_bounded_waits_time_out_and_the_context_recovers():
     torch.cuda.synchronize()
     np.testing.assert_array_equal(np.tril(host(G)), np.tril(host(G_ref)))
     prob.close()
+
+
+def test_layered_passes_time_out_and_recover():
+    """The passes over many points wait for tensor-core products in every precision.  With none issued:
+    calls that synchronise return GN_ERR_TIMEOUT and leave theta alone; gn_jacobian and gn_gradient only launch,
+    leave no entry unwritten, and the next call that synchronises reports them, once."""
+    from paper_2509_14185_gb300 import gn
+    from paper_2509_14185_gb300 import inputs as I
+    L = gn.lib()
+    n = 2100
+    w = I.small_case(I.IPM, [2, 48, 48, 48, 2], n, n_bnd=30, seed=3)
+    prob, ref = gpu_problem(w), gpu_problem(w)
+    Pp, th = prob.P + 1, dev(w.theta)
+    J0, g0 = ref.jacobian(th, w.lam), ref.gradient(th, w.lam)
+    loss0 = ref.gn_residual(th, w.lam)[1]
+    J = torch.full_like(J0, 7.0)
+    g = prob.new_vec(Pp)
+    A = torch.eye(Pp, dtype=torch.float64, device="cuda")
+    delta, out = prob.new_vec(Pp), ctypes.c_double(0.0)
+
+    def step(p, theta, call=L.gn_step):
+        lam, gam = ctypes.c_double(w.lam), ctypes.c_double(1e-2)
+        return call(p.h, gn._ptr(theta), ctypes.byref(lam), ctypes.byref(gam), None), lam.value, gam.value
+
+    torch.cuda.synchronize()
+    try:
+        assert L.gn_test_bounded_waits(20_000_000, 1) == 0
+        assert L.gn_residual(prob.h, gn._ptr(th), w.lam, None, ctypes.byref(out)) == GN_ERR_TIMEOUT
+        assert L.gn_max_residual(prob.h, gn._ptr(th), w.lam, ctypes.byref(out)) == GN_ERR_TIMEOUT
+        assert L.gn_jacobian(prob.h, gn._ptr(th), w.lam, gn._ptr(J), J.stride(0), 0, J.shape[0]) == 0
+        assert L.gn_gradient(prob.h, gn._ptr(th), w.lam, None, gn._ptr(g)) == 0
+    finally:
+        assert L.gn_test_bounded_waits(0, 0) == 0
+    torch.cuda.synchronize()
+    off = 2 * 48 + 48
+    for i, o in ((48, 48), (48, 48)):
+        assert bool(torch.isnan(J[:2 * n, off:off + i * o]).all())
+        off += i * o + o
+    assert bool(torch.isnan(g).any())
+    assert prob.gn_damped_solve(A, g0, 1.0, delta)[0] == GN_ERR_TIMEOUT     # reported
+    assert prob.gn_damped_solve(A, g0, 1.0, delta)[0] == 0                  # and cleared
+    theta, theta_ref = dev(w.theta), dev(w.theta)
+    pg = gpu_problem(w)
+    try:
+        assert L.gn_test_bounded_waits(20_000_000, 1) == 0
+        assert step(prob, theta)[0] == GN_ERR_TIMEOUT
+        assert step(pg, theta, L.gn_step_graph) == (GN_ERR_TIMEOUT, w.lam, 1e-2)
+    finally:
+        assert L.gn_test_bounded_waits(0, 0) == 0
+    np.testing.assert_array_equal(host(theta), w.theta)
+    # undisturbed again
+    assert prob.gn_residual(th, w.lam) == (0, loss0)
+    assert torch.equal(prob.jacobian(th, w.lam), J0) and torch.equal(prob.gradient(th, w.lam), g0)
+    assert step(prob, theta) == step(ref, theta_ref) and torch.equal(theta, theta_ref)
+    for p in (prob, ref, pg):
+        p.close()
