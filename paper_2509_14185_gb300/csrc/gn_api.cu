@@ -758,13 +758,13 @@ int gn_set_gram_tile(gn_handle* h, int tile_n) {
 
 int gn_gram_tile_choice(const gn_handle* h, int64_t nrows, int* tile_n) {
   if (!h || !tile_n || nrows < 0) return GN_ERR_INVALID;
-  *tile_n = h->gram_tile > 0 ? h->gram_tile : gram_tile_choice(h->n_slices, h->Pp, nrows);
+  *tile_n = gram_tile_choice(h, nrows);
   return GN_OK;
 }
 
 int gn_gram_split_choice(const gn_handle* h, int64_t nrows, int* ksplit) {
   if (!h || !ksplit || nrows < 0) return GN_ERR_INVALID;
-  *ksplit = h->gram_ksplit > 0 ? h->gram_ksplit : gram_split_choice(h->n_slices, h->Pp, nrows);
+  *ksplit = gram_split_choice(h, nrows);
   return GN_OK;
 }
 

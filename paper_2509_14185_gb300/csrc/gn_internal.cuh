@@ -246,8 +246,8 @@ struct GraphKey {
 };
 size_t chol_split_ws_bytes(int64_t n, int S);
 // split-K factor and tile width the Gram autotuner recorded for this shape (0: not tuned yet)
-int gram_split_choice(int S, int64_t Pp, int64_t nrows);
-int gram_tile_choice(int S, int64_t Pp, int64_t nrows);
+int gram_split_choice(const gn_handle* h, int64_t nrows);
+int gram_tile_choice(const gn_handle* h, int64_t nrows);
 cudaError_t ensure_chol_streams(gn_handle* h);
 void graph_release(gn_handle* h);
 // wait for the handle's stream; GN_ERR_TIMEOUT if a bounded wait has run out since the last report

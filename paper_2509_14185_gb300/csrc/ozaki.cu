@@ -1051,15 +1051,6 @@ int tune(gn_handle* h, int S, const OzOperand& op, int64_t nrows, double* C, voi
 }
 }  // namespace
 
-int gram_split_choice(int S, int64_t Pp, int64_t nrows) {
-  GramChoice ch;
-  return lookup(S, Pp, nrows, &ch) ? ch.ks : 0;
-}
-int gram_tile_choice(int S, int64_t Pp, int64_t nrows) {
-  GramChoice ch;
-  return lookup(S, Pp, nrows, &ch) ? ch.tn : 0;
-}
-
 // Six slices without a forced tile or split go by residues (crt.cu): fewer products, and exact.
 // Not when its workspace could not be had, nor for a wide G of few rows, where writing and
 // reconstructing 13 residues per entry costs more than the products save.  Best slice products /
@@ -1072,11 +1063,6 @@ bool by_residues(const gn_handle* h, int64_t nrows) {
 size_t colmax_bytes(int64_t Pp) { return (size_t)CM_CHUNKS * rup(Pp, TM) * 8 + 256; }
 size_t residue_bytes(const gn_handle* h, int64_t nrows) {
   return crt_plan(h->Pp, nrows).bytes + colmax_bytes(h->Pp);
-}
-// the choice the gn_gram_*_choice calls report for a shape that goes by residues
-void record_default_choice(const gn_handle* h, int64_t nrows) {
-  std::lock_guard<std::mutex> g(g_tune_mu);
-  g_tune.emplace(std::make_tuple(h->n_slices, (h->Pp + TM - 1) / TM, gram_chunks(nrows)), GramChoice());
 }
 // Does a Gram of nrows rows go by residues?  No memory for the planes is remembered (the slices have
 // to do from then on); any other failure is the caller's.
@@ -1097,16 +1083,28 @@ size_t slice_bytes(gn_handle* h, int64_t nrows) {
 }
 }  // namespace
 
+// What gn_gram_split_choice and gn_gram_tile_choice report (0: not tuned yet).  The table of tuned choices is
+// the slices' own: residues have neither a split nor a choice of tiles.
+int gram_split_choice(const gn_handle* h, int64_t nrows) {
+  GramChoice ch;
+  if (h->gram_ksplit > 0) return h->gram_ksplit;
+  if (by_residues(h, nrows)) return 1;
+  return lookup(h->n_slices, h->Pp, nrows, &ch) ? ch.ks : 0;
+}
+int gram_tile_choice(const gn_handle* h, int64_t nrows) {
+  GramChoice ch;
+  if (h->gram_tile > 0) return h->gram_tile;
+  if (by_residues(h, nrows)) return TN;
+  return lookup(h->n_slices, h->Pp, nrows, &ch) ? ch.tn : 0;
+}
+
 // Tune the Gram of the handle's largest row block ahead of a capture, on a zeroed operand
 // (tensor-core time does not depend on the values).
 int pretune_gram(gn_handle* h) {
   if (h->precision == GN_PREC_FP64 || h->gram_ksplit > 0 || h->gram_tile > 0 || h->n_rows <= 0) return GN_OK;
   const int S = h->n_slices;
   const int64_t nrows = h->jrows;
-  if (by_residues(h, nrows)) {
-    record_default_choice(h, nrows);
-    return GN_OK;
-  }
+  if (by_residues(h, nrows)) return GN_OK;
   GramChoice ks;
   if (lookup(S, h->Pp, nrows, &ks)) return GN_OK;
   const size_t opb = oz_operand_bytes(S, h->Pp, nrows);
@@ -1172,7 +1170,6 @@ int split_gram(gn_handle* h, const double* J, int64_t ld, int64_t nrows, double*
         rc = crt_product(pl, k, h->Pp, h->split_ws, G, h->Pp, accumulate || k0 > 0, 0, -1, 0, 0, h->flag + 2, h->st);
       if (rc) return rc;
     }
-    record_default_choice(h, nrows);
     return GN_OK;
   }
   const size_t opb = oz_operand_bytes(S, h->Pp, nrows);
@@ -1204,7 +1201,7 @@ int64_t pipeline_chunk_tiles(gn_handle* h) {
   if (h->pipe_tiles == 0 || h->precision != GN_PREC_SPLIT_ALL || h->n_rows <= 0) return 0;
   if ((h->n_rows + h->jrows - 1) / h->jrows != 1) return 0;
   GramChoice ch;   // the pipeline's column chunks use square tiles without split-K
-  if (!gram_choice(h, h->n_rows, &ch)) {
+  if (!by_residues(h, h->n_rows) && !gram_choice(h, h->n_rows, &ch)) {
     ch.ks = h->gram_ksplit > 0 ? h->gram_ksplit : 1;
     ch.tn = h->gram_tile > 0 ? h->gram_tile : TN;
   }

@@ -84,3 +84,18 @@ def test_forced_tiles_keep_the_slice_products():
     G64 = torch.tril(_gram(p, J, 500))
     assert p.gn_gram_tile_choice(500) == 64
     assert float((G6 - ref).norm()) <= float((G64 - ref).norm())
+
+
+def test_residues_leave_the_table_of_tuned_slices_alone():
+    """544 rows of 2114 columns go by residues, 520 (as many chunks of the contraction) by slices: what
+    one reports or records does not reach the other."""
+    p, n = _problem([44, 44])
+    assert n == 2114
+    p.gn_set_precision(1, 6)
+    J = torch.randn(544, n, generator=torch.Generator(device="cuda").manual_seed(2), dtype=torch.float64, device="cuda")
+    assert (p.gn_gram_split_choice(544), p.gn_gram_tile_choice(544)) == (1, 128)
+    _gram(p, J, 544)
+    assert (p.gn_gram_split_choice(520), p.gn_gram_tile_choice(520)) == (0, 0)      # not tuned yet
+    _gram(p, J[:520], 520)
+    assert p.gn_gram_split_choice(520) >= 1 and p.gn_gram_tile_choice(520) in (64, 128)
+    assert (p.gn_gram_split_choice(544), p.gn_gram_tile_choice(544)) == (1, 128)
