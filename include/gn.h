@@ -80,8 +80,12 @@ enum gn_equation {
                          (V = (1+lambda) y + U, U = (d2 Psi, -d1 Psi))                    */
 };
 
-/* Precision of the Gram product G = J~^T J~ (Methods, "Second-order Optimizer";
- * everything else is always FP64). */
+/* Precision of the Gram product G = J~^T J~ (Methods, "Second-order Optimizer").  Residuals,
+ * Jacobian rows and gradients have FP64's accuracy in every mode.  For many points (2048 in 2D, 4096 in 1D;
+ * tanh networks of two and more hidden layers, all of them 24 to 64 wide, 32 for Jacobian rows) the sums
+ * over a hidden layer's width, and in 2D over a Jacobian entry's terms, are formed on the tensor cores
+ * from 62-bit operands: each is off by no more than an FP64 sum of its n terms may be, n 2^-53 times the
+ * sum of the terms' magnitudes, and is summed in FP64 where the operands' scales do not allow that. */
 enum gn_precision {
   GN_PREC_FP64 = 0,        /* native FP64 (DFMA) Gram */
   GN_PREC_SPLIT_BF16 = 1,  /* Ozaki split: each FP64 column of J~ scaled by a power of two and
@@ -89,7 +93,11 @@ enum gn_precision {
                               tensor cores with exactly representable FP32 partial sums,
                               combined in double-FP32 and returned as FP64.  With six slices the
                               Gram takes the same 48-bit operands by their residues modulo 13
-                              coprime numbers instead: the exact integer product, rounded once */
+                              coprime numbers instead: the exact integer product, rounded once.
+                              Its planes take more memory than the slices (4.7 against 1.7 GB at
+                              16385 x 8514; at most the larger of the slices' and 6 GB, and 1 GB);
+                              a handle that cannot have it keeps to the slices from then on, which
+                              gn_gram_split_choice and gn_gram_tile_choice show */
   GN_PREC_SPLIT_ALL = 2    /* as GN_PREC_SPLIT_BF16, and the other two dense contractions too:
                               the CCF Hilbert contraction J_U = K J_g and the trailing updates
                               of the blocked Cholesky factorisation (accumulated in double-FP32;
@@ -199,7 +207,8 @@ typedef struct gn_handle gn_handle;
 
 /* Create a handle for one profile fit.  Copies *p (the point arrays stay
  * borrowed), allocates all device workspace (J~, G, factor, vectors, the CCF
- * Hilbert matrix) on the current device, and binds the handle to
+ * Hilbert matrix; for many points up to about 320 MB for their passes, without
+ * which they run one warp per point) on the current device, and binds the handle to
  * cuda_stream (a cudaStream_t; NULL = legacy default stream).
  * Cites: problem statement in Methods ("Self-similar Solutions", "Solution
  * Modeling", "Training Loss").  Errors: GN_ERR_INVALID, GN_ERR_OOM, GN_ERR_CUDA. */

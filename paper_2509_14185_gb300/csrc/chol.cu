@@ -1217,20 +1217,22 @@ size_t chol_split_ws_bytes(int64_t n, int S) {
 // the deferred bulk updates in the middle, and the pipelined step's Gram chunks at the lowest
 // (numerically greater is lower; with fewer levels neighbours share one).
 cudaError_t ensure_chol_streams(gn_handle* h) {
-  if (h->st_hi) return cudaSuccess;
+  if (h->chol_streams) return cudaSuccess;
   int least = 0, greatest = 0;
   cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
   const int middle = greatest + (least - greatest + 1) / 2;
   const int next = greatest < middle ? greatest + 1 : greatest;
-  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_hi, cudaStreamNonBlocking, greatest);
-  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_up, cudaStreamNonBlocking, next);
-  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_lo, cudaStreamNonBlocking, middle);
-  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->st_g, cudaStreamNonBlocking, least);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_panel, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_rest, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_next, cudaEventDisableTiming);
-  for (cudaEvent_t& b : h->ev_bulk)
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b, cudaEventDisableTiming);
+  // (what an earlier, failed call created is kept)
+  auto stream = [&](cudaStream_t* s, int priority) {
+    if (e == cudaSuccess && !*s) e = cudaStreamCreateWithPriority(s, cudaStreamNonBlocking, priority);
+  };
+  stream(&h->st_hi, greatest);
+  stream(&h->st_up, next);
+  stream(&h->st_lo, middle);
+  stream(&h->st_g, least);
+  for (cudaEvent_t* v : {&h->ev_panel, &h->ev_rest, &h->ev_next, &h->ev_bulk[0], &h->ev_bulk[1]})
+    if (e == cudaSuccess && !*v) e = cudaEventCreateWithFlags(v, cudaEventDisableTiming);
+  h->chol_streams = e == cudaSuccess;
   return e;
 }
 

@@ -167,6 +167,7 @@ int run_pass(gn_handle* h, const double* theta, double lam, const Pass& ps, doub
   if (ps.mode == MODE_GRADIENT) {
     JetArgs b = a;
     b.kind = KIND_INTERIOR;
+    b.mode = MODE_GRADIENT;
     b.n = n;
     const bool layered = takes_layers(h, b);
     side = side && layered && h->eq != GN_CCF && h->p.n_d1 == 0 && h->p.n_d2 == 0;

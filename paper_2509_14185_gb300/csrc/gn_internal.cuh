@@ -150,6 +150,7 @@ struct gn_handle {
   double* ema_ws = nullptr;
   int64_t ema_len = 0;
   // streams of the factorisations' look-ahead (created on first use)
+  bool chol_streams = false;      // all of them, and the events, exist
   cudaStream_t st_hi = nullptr;   // critical path (highest priority)
   cudaStream_t st_up = nullptr;   // updates of the next columns (next priority)
   cudaStream_t st_lo = nullptr;   // deferred bulk updates (middle priority)

@@ -1163,9 +1163,9 @@ cudaError_t run_gemm(const LayArgs& a, cudaStream_t st) {
 
 // lay_hidden_entries always computes two rows by 64 outputs by 64 columns (and stops at the narrower
 // layer's columns); the FP64 form pays for what there is.  Jacobian, FP64 -> products, three hidden layers, 8192
-// points.  Two rows per point: width 40 1.96 -> 1.98 ms, 44 2.08 -> 2.04, 52 2.30 -> 2.11, 64 2.61 -> 2.20.
-// Three rows (every second pair half empty): 52 3.11 -> 3.19 ms, 56 3.27 -> 3.26, 60 3.45 -> 3.31,
-// 64 3.57 -> 3.31; 2048 points cross at the same widths.  A single row leaves half of every product empty.
+// points.  Two rows per point: width 40 1.96 -> 1.94 ms, 44 2.09 -> 2.01, 52 2.32 -> 2.10, 64 2.67 -> 2.27.
+// Three rows (every second pair half empty): 52 3.13 -> 3.17 ms, 56 3.30 -> 3.30, 60 3.51 -> 3.35, 64 3.65 -> 3.42.
+// A single row leaves half of every product empty.
 template <int D>
 bool hidden_entries(const NetDesc& net, int nr) {
   bool wide = D == 2 && nr > 1;
@@ -1369,28 +1369,42 @@ cudaError_t layers_mode(const JetArgs& a, void* ws, size_t bytes, cudaStream_t s
 
 }  // namespace
 
-// The layered path takes tanh networks of at least two hidden layers, none wider than the 64
-// columns of its tiles or narrower than 24, and point sets (all of them, not a row block's, so that
-// a block's rows equal the whole's) of 2048 points in 2D, 4096 in 1D.  Below that its chain of
-// 2 L launches takes longer than one pointwise kernel.  Pointwise / layered time, residual and
-// Jacobian pass: 1D width 32 x 2, 2048 points 44 / 54 and 79 / 111 us, 4096 points 79 / 58 and 147 / 133;
-// 1D 64 x 3, 8192 points 390 / 128 and 1120 / 541; 2D IPM 32 x 2, 1024 points 54 / 58 and 142 / 196, 2048 points
-// 106 / 62 and 304 / 282; IPM 64 x 3, 8192 points 1170 / 260 and 5119 / 2619.  Width 16 x 3, IPM, 8192 points:
-// 332 / 181 and 911 / 1063 (the products are padded to 64 columns).
+// The layered path takes tanh networks of at least two hidden layers, none wider than the 64 columns of its
+// tiles, and point sets (all of them, not a row block's, so that a block's rows equal the whole's) large enough
+// for its chain of 2 L launches and wide enough for what its tiles pad.  Pointwise / layered time in us over 2, 3 and 4
+// hidden layers (FP64, Burgers and IPM; Boussinesq gains more than IPM):
+//   1D residual   24 wide 4096 points 76/76 92/102 111/129, 6000 104/78 131/102 158/129; 32 wide 4096 82/64 102/92 127/119
+//   1D Jacobian   28 wide 16384 points 455/409 653/668 852/909; 32 wide 4096 149/141 217/225 285/303, 6000 217/164
+//                 317/254 416/352; 40 wide 4096 244/176 389/278 532/377
+//   1D gradient   24 wide 16384 points 502/497 707/720 913/946; 28 wide 4096 221/190 307/262 395/333
+//   2D residual   24 wide 1024 points 51/63 61/88 70/113, 2048 98/67 121/92 143/117
+//   2D Jacobian   24 wide 8192 points 827/876 1223/1292 1656/1786; 32 wide 2048 309/295 477/436 647/614
+//   2D gradient   24 wide 1024 points 201/215 269/284 337/348, 2048 314/247 426/333 541/414
+// and at 64 wide, 3 hidden layers, 8192 points: Burgers 391/137 1134/557 1760/661, IPM 1177/297 5123/2273 4389/1722.
 static bool layers_net(const NetDesc& net) {
   if (net.fourier || net.exp_out || net.L < 3) return false;
   for (int l = 1; l < net.L; l++)
     if (net.w[l] > kLayW || net.w[l] < 24) return false;
   return true;
 }
-static int64_t layers_min_points(int d) { return d == 1 ? 4096 : 2048; }
+static int64_t layers_min_points(const NetDesc& net, int mode) {
+  const int d = net.w[0];
+  int w = kLayW;   // the narrowest hidden layer
+  for (int l = 1; l < net.L; l++) w = net.w[l] < w ? net.w[l] : w;
+  if (w < (mode == MODE_JACOBIAN ? 32 : mode == MODE_GRADIENT && d == 1 ? 28 : 24)) return INT64_MAX;
+  if (d == 2) return 2048;
+  return mode != MODE_GRADIENT && w < (mode == MODE_JACOBIAN ? 40 : 32) ? 5000 : 4096;
+}
 
 bool layers_eligible(const JetArgs& a) {
-  return a.kind != KIND_PROBE && a.n >= layers_min_points(a.net.w[0]) && layers_net(a.net);
+  return a.kind != KIND_PROBE && layers_net(a.net) && a.n >= layers_min_points(a.net, a.mode);
 }
 
 size_t layers_ws_bytes(const NetDesc& net, int d, int nf, int ne, int64_t npt) {
-  if (npt < layers_min_points(d) || !layers_net(net)) return 0;
+  bool any = false;
+  for (int mode : {MODE_RESIDUAL, MODE_JACOBIAN, MODE_GRADIENT})
+    any = any || (layers_net(net) && npt >= layers_min_points(net, mode));
+  if (!any) return 0;
   const int64_t per = lay_point_doubles(net, d, nf, ne, MODE_JACOBIAN) * 8;
   const int64_t cap = (int64_t)320 << 20;
   return (size_t)(kLayFixed + lay_parts_doubles(net) * 8 + (per * npt < cap ? per * npt : cap));

@@ -252,3 +252,30 @@ def test_entries_of_a_constant_neuron(name, hidden):
         ref = bias * np.tanh(b)
         assert bool((ref != 0).any())
         assert bool(((entry - ref).abs() <= 15 * 2.0 ** -53 * ref.abs()).all())
+
+
+@pytest.mark.parametrize("name,hidden,n,call,layered", [
+    ("burgers", [24] * 4, 4999, "residual", False), ("burgers", [24] * 4, 5000, "residual", True),
+    ("burgers", [32, 40], 4095, "residual", False), ("burgers", [32, 40], 4096, "residual", True),
+    ("burgers", [64, 31], 9000, "jacobian", False), ("burgers", [39, 64], 4999, "jacobian", False),
+    ("burgers", [32, 64], 5000, "jacobian", True), ("burgers", [40, 64], 4096, "jacobian", True),
+    ("burgers", [27, 64], 9000, "gradient", False), ("burgers", [28, 64], 4096, "gradient", True),
+    ("ipm", [24, 24], 2047, "residual", False), ("ipm", [24, 24], 2048, "residual", True),
+    ("ipm", [64, 31], 3000, "jacobian", False), ("ipm", [64, 32], 2048, "jacobian", True),
+    ("ipm", [64, 24], 2048, "gradient", True), ("ipm", [64, 23], 3000, "gradient", False)])
+def test_route_by_width_and_points(name, hidden, n, call, layered):
+    """Narrow networks and few points stay with the one-warp-per-point kernel where it is the faster one:
+    the weights' transposition, the interior and the normalisation point (and a gradient's sum)."""
+    from paper_2509_14185_gb300 import gn
+    eq, nf = EQS[name]
+    w = I.small_case(eq, [I.EQUATION_DIM[eq]] + hidden + [nf], n, n_bnd=0)
+    p = gpu_problem(w)
+    th = dev(w.theta)
+    out = {"residual": lambda: p.gn_residual(th, w.lam, r, want_loss=False), "jacobian": lambda: p.jacobian(th, w.lam),
+           "gradient": lambda: p.gradient(th, w.lam)}
+    r = p.new_vec(p.n_rows)
+    k = gn.lib().gn_kernel_launches()
+    out[call]()
+    k = gn.lib().gn_kernel_launches() - k
+    torch.cuda.synchronize()
+    assert (k > 5) == layered, k
