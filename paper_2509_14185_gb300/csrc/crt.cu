@@ -22,8 +22,8 @@
 // and of B per 64-wide K stage), two 256-column accumulators so that one chunk's products run while
 // the last is reduced, persistent pairs over the (modulus, tile) items.  It wants the full shared-memory
 // bandwidth (64 bytes per clock of operand reads, 64 of copies), so its waits suspend instead of polling
-// (tc.cuh) and its loops keep to the 512 clocks of a stage.  8514 columns, 16385 rows: 10.6 ms = 1.57 PFLOP/s,
-// tensor pipe 0.66 busy (0.71 with four times fewer reductions); first version 16.9 ms.  Clusters of two pairs
+// (tc.cuh) and its loops keep to the 512 clocks of a stage.  8514 columns, 16385 rows: 10.6 ms = 1.57 PFLOP/s
+// (2501 rows of 4850 columns: tensor pipe 57 % busy); first version 16.9 ms.  Clusters of two pairs
 // sharing B by multicast cut the L2 reads by a fifth and took 11.8 ms: they fill only 144 of the 152 SMs.
 // Whole Gram, slices -> residues: 16.84 -> 13.35 ms there (0.17 column maxima, 1.14 residues, 10.6 products, 0.46
 // reconstruction), 1154 x 4097 0.303 -> 0.211 ms, 322 x 1025 0.110 -> 0.066 ms; error against 64 bits 3e-10 -> 2.6e-15 (the

@@ -825,8 +825,8 @@ __global__ void __launch_bounds__(256) lay_entries(const LayEntries p) {
 // 0.05 to 0.4 % of them), or with a factor that is not finite, is summed in FP64.  (Its operands stay in shared
 // memory for that: a warp in sixteen has such an entry, and all wait for the slowest.)
 // Bound by the digits and the 64-bit recombination (integer pipes) and by J's stores.
-// Jacobian of 32,768 IPM rows, four hidden layers of 64: 6.96 -> 5.54 ms.  Digits dealt over all threads
-// (5.64 ms) and stores of the unit before beside the products (5.67 ms) were no faster.
+// Jacobian of 8192 IPM points, three hidden layers of 64, FP64 form -> products: 2.67 -> 2.27 ms; 32,768 rows of four
+// layers take 5.73 ms.  Digits dealt over all threads and stores of the unit before beside the products were 2 % slower.
 constexpr int kEntS = 8;
 constexpr int kEntASlice = 128 * 64, kEntBSlice = 64 * 64;   // K padded to 32: the layout of lay_gemm
 constexpr int kEntOps = kEntS * (kEntASlice + kEntBSlice);
